@@ -20,16 +20,17 @@
 // whose level bounds stay on the device, so the levels need no host round
 // trip; each node of the last prefix level is then searched depth-first by one
 // thread, unless the prefix already reaches size K - 1 and one more
-// warp-parallel step ends it.  In LOOP mode the prefix stops at size K - 2:
+// warp-parallel step ends it.  In LOOP mode the prefix stops at size K - 3:
 // the bond that completes a cluster of size K joins two vertices the set
-// already has, so a node of size K - 2 finds both remaining sizes in one
+// already has, so a set of size K - 2 finds both remaining sizes in one
 // warp-parallel step (each lane's child, then the child's closing bonds among
-// the node's later candidates) and the far more numerous sets of size K - 1
-// that cannot be closed are never stored; a child of size K - 2 is kept only
-// if two more candidate bonds can still close it (closable2).  Every unit
-// first counts what it emits per cluster size; an exclusive scan over (size,
-// unit) gives each unit its output slots, and a second pass writes.  The
-// output is grouped by size and deterministic.
+// the set's later candidates), and a node of size K - 3 does this for each of
+// its children in turn, in shared memory: neither the sets of size K - 2 nor
+// the far more numerous ones of size K - 1 are ever stored.  A child of size
+// K - 2 is looked at only if two more candidate bonds can still close it
+// (closable2).  Every unit first counts what it emits per cluster size; an
+// exclusive scan over (size, unit) gives each unit its output slots, and a
+// second pass writes.  The output is grouped by size and deterministic.
 //
 // Terms (Eq. A4): a term is a set of pairwise vertex-disjoint clusters with
 // total size <= K (the connected components of one P/Q string).  Tuples
@@ -315,6 +316,16 @@ __global__ void row_starts_kernel(const int64_t *scanned, int rows, int64_t cols
     starts[r] = (r == rows || at >= n) ? *total : scanned[at];
 }
 
+// The first output slot of every size from the scanned three-row table of the
+// closing step: size q <= K - 2 starts with level q - 1 of row 0, sizes K - 1
+// and K with rows 1 and 2; starts[K + 1] is the total.
+__global__ void close_starts_kernel(const int64_t *scanned, int64_t cap, const int64_t *lv, int K, int64_t *starts,
+                                    const int64_t *total)
+{
+    const int q = threadIdx.x;
+    if (q > K + 1) return;
+    starts[q] = q <= 2 ? 0 : (q <= K - 2 ? scanned[lv[q - 2]] : (q <= K ? scanned[(q - K + 2) * cap] : *total));
+}
 
 // ---------------------------------------------------------------- search arena
 // Every prefix level lives in one node arena: level d (d = 1: the anchors,
@@ -322,7 +333,13 @@ __global__ void row_starts_kernel(const int64_t *scanned, int rows, int64_t cols
 // device, so the levels are expanded without a host round trip.  A level
 // whose children would not fit stops the search (ctl->stop = d, ctl->need =
 // the size it asked for) and every deeper level is left empty.  Count and
-// slot tables are [K+1][cap], indexed by arena position.
+// slot tables are [K+1][cap], indexed by arena position; with the closing
+// step (LOOP mode, K >= 4) a node of level t emits size t + 1 only, except
+// the last level's, which emit sizes K - 2, K - 1 and K, so three rows hold
+// the counts in output order: row 0 every level's own size (levels ascend
+// with the arena position), rows 1 and 2 the last level's K - 1 and K.  On
+// the 16 x 16 lattice at K = 8 that is a table of 3 x 7,168 entries to clear
+// and scan instead of 9 x 11,264.
 struct SearchCtl {
     int32_t cand_overflow;        // a candidate list outgrew kNodeU
     int32_t stop;                 // first level whose children did not fit (0: none)
@@ -336,9 +353,9 @@ struct Arena {
     int32_t *child_cnt;           // [cap] children per node
     int64_t *child_off;           // [cap] child offset within the node's chunk
     int64_t *chunk_tot;           // [grid] children per chunk, then their exclusive scan
-    int32_t *counts;              // [K+1][cap] clusters emitted per (size, node)
+    int32_t *counts;              // [K+1][cap] clusters emitted per (size, node); [3][cap] with the closing step
     uint64_t *gmask, *emask;      // [cap] per node: candidates that make a child / an emitted cluster
-    const int64_t *base;          // [K+1][cap] first output slot per (size, node)
+    const int64_t *base;          // as counts: first output slot per (size, node)
     SearchCtl *ctl;
 };
 
@@ -398,10 +415,10 @@ __global__ void roots_kernel(GeomView g, int n_closed, int mode, Arena A, Emit o
 //   kEmitCount: emissions only (the last level)
 //   kChildren:  write the children of level lo == hi, unless the search stopped
 //   kEmit:      write the emitted clusters of levels lo..hi
-//   kPairCount: the closing level of LOOP mode (nodes of size K - 2): sizes
-//               K - 1 and K counted together, no nodes of size K - 1 made
-//               (see pair_node)
-enum ExpandPass { kCount = 0, kChildren = 1, kEmit = 2, kEmitCount = 3, kPairCount = 4 };
+//   kClose:     the last level of LOOP mode (nodes of size K - 3): sizes K - 2,
+//               K - 1 and K counted together, no nodes of size K - 2 or K - 1
+//               made (see close_child)
+enum ExpandPass { kCount = 0, kChildren = 1, kEmit = 2, kEmitCount = 3, kClose = 4 };
 constexpr int kExpandWarps = 4;
 constexpr int kMaxNew = kNodeU / (kPrefixMax + 1);   // new candidates per step (site degree - 1)
 constexpr int kNodeWords = (int)(sizeof(Node) / 4);
@@ -559,23 +576,25 @@ __device__ __forceinline__ void sort_regs(int32_t (&x)[N])
         }
 }
 
-// Writes the cluster S + e1 (+ e2 when >= 0) of a node: bonds and vertices
-// (the node's list plus b when >= 0) sorted ascending, rows padded with -1.
-__device__ void write_child_cluster(const Emit &o, int64_t slot, const Node &nd, int e1, int e2, int b)
+// Writes the cluster S + e0 (+ e1, e2 when >= 0) of a node: bonds and vertices
+// (the node's list plus b0, b1 when >= 0) sorted ascending, rows padded with -1.
+__device__ void write_child_cluster(const Emit &o, int64_t slot, const Node &nd, int e0, int e1, int e2, int b0, int b1)
 {
-    constexpr int NS = kPrefixMax + 2, NVx = kNodeV + 1;
+    constexpr int NS = kPrefixMax + 3, NVx = kNodeV + 2;
     const int t = nd.t, vn = nd.vn;
     int32_t sv[NS], vv[NVx];
 #pragma unroll
     for (int q = 0; q < kPrefixMax; ++q) sv[q] = q < t ? nd.S[q] : INT_MAX;
-    sv[kPrefixMax] = e1;
-    sv[kPrefixMax + 1] = e2 >= 0 ? e2 : INT_MAX;
+    sv[kPrefixMax] = e0;
+    sv[kPrefixMax + 1] = e1 >= 0 ? e1 : INT_MAX;
+    sv[kPrefixMax + 2] = e2 >= 0 ? e2 : INT_MAX;
 #pragma unroll
     for (int q = 0; q < kNodeV; ++q) vv[q] = q < vn ? nd.vv[q] : INT_MAX;
-    vv[kNodeV] = b >= 0 ? b : INT_MAX;
+    vv[kNodeV] = b0 >= 0 ? b0 : INT_MAX;
+    vv[kNodeV + 1] = b1 >= 0 ? b1 : INT_MAX;
     sort_regs(sv);
     sort_regs(vv);
-    const int s = t + 1 + (e2 >= 0 ? 1 : 0), n = vn + (b >= 0 ? 1 : 0);
+    const int s = t + 1 + (e1 >= 0 ? 1 : 0) + (e2 >= 0 ? 1 : 0), n = vn + (b0 >= 0 ? 1 : 0) + (b1 >= 0 ? 1 : 0);
     int32_t *er = o.edges + slot * o.width;
 #pragma unroll
     for (int q = 0; q < NS; ++q)
@@ -589,93 +608,121 @@ __device__ void write_child_cluster(const Emit &o, int64_t slot, const Node &nd,
     o.size[slot] = s;
 }
 
-// A node of size K - 2 in LOOP mode, both remaining levels at once.  Its child
-// S + U[i] (size K - 1) is a cluster iff it has no degree-one vertex; a
-// cluster of size K below that child is S + U[i] + U[j] with a bond U[j] of
-// the child's candidate list that removes every degree-one vertex without
-// adding one: both ends of U[j] already belong to the child, so U[j] is not
-// one of the child's new candidates (those lead off the child's vertex set)
-// and is a later candidate U[j], j > i, of this node.  It closes the child
-// iff its ends include every degree-one vertex of the child (there are at
-// most two).  The sizes K - 1 and K come out in the order of the level-by-
-// level search: child by child, and per child in candidate order.
-//   counting (kPairCount): per node the size K - 1 and size K counts, the
-//     lanes with an emitted child (emask) and with a closing bond (gmask)
-//   writing (kEmit): both sizes, from the slots of the (size, node) scan
-// `want` is the lane mask of the writing pass.
-template <int PASS>
-__device__ void pair_node(const Arena &A, const Node &nd, int64_t u, const NodeTabs &T, uint32_t node_dmask,
-                          uint64_t want, const Emit &out)
+// A child of size K - 2 of a node of size K - 3 in LOOP mode, both remaining
+// levels at once.  The grandchild, the child's set + V[i] (size K - 1; V the
+// child's candidate list), is a cluster iff it has no degree-one vertex; a
+// cluster of size K below it adds a bond V[j] that removes every degree-one
+// vertex without adding one: both ends of V[j] already belong to the
+// grandchild, so V[j] is not one of its new candidates (those lead off its
+// vertex set) and is a later candidate V[j], j > i.  It closes the grandchild
+// iff its ends include every degree-one vertex (there are at most two).  The
+// sizes K - 1 and K come out in the order of the level-by-level search:
+// grandchild by grandchild, and per grandchild in candidate order.
+//
+// The whole warp works on one child: its candidates are the node's later ones
+// and the new ones, a lane each (two rounds above 32), and the closing bonds
+// of a lane are the bits of an and of candidate masks -- the candidates with
+// both ends in the set, those at each degree-one vertex (at most four, by
+// closable2), those sharing the lane's outside end -- so the step costs a few
+// ballots per child, not a walk over the list per lane.  Building the child
+// here instead of storing it as a node of the arena saves its 320 bytes
+// written and read again and one launch: 8 x 8 x 8, K = 10 has 3.1 M nodes up
+// to size 7 and would store 1.7 M of size 8, which did not fit the largest
+// arena, so sizes 8 to 10 were searched depth-first, a thread per node (92 of
+// the 112 ms of a pass with three tensor sets; now 15.8 ms).  At K = 8 on
+// 16 x 16 (3.6 k nodes of size 5) the pass goes from 0.698 to 0.671 ms.
+struct CloseTabs {
+    int32_t *e, *o, *ia, *ib;     // V[q], its end outside the child (-1: none), the ends' indices in the child
+    int32_t *nu;                  // the new candidates of the child at hand
+};
+
+template <bool WRITE>
+__device__ void close_child(const GeomView &g, const Node &nd, const NodeTabs &T, const CloseTabs &C, int io, int cb,
+                            uint32_t cdm, int nn, int64_t slotA, int64_t slotB, int &nA, int &nB, const Emit &out)
 {
-    constexpr int pass = PASS;
     const int lane = threadIdx.x & 31;
     const unsigned lt = (1u << lane) - 1u;
-    const int nU = nd.nU, t = nd.t;
-    int n_emit = 0, n_pair = 0;
-    uint64_t emask = 0, pmask = 0;
-    const int64_t ebase = (pass == kEmit) ? A.base[(int64_t)(t + 1) * A.cap + u] : 0;
-    const int64_t pbase = (pass == kEmit) ? A.base[(int64_t)(t + 2) * A.cap + u] : 0;
-    for (int i0 = 0; i0 < nU; i0 += 32) {
+    const int vn = nd.vn, m0 = nd.nU - io - 1, n = m0 + nn;
+    for (int q = lane; q < n; q += 32) {
+        int e, x, y, ia, ib;
+        if (q < m0) {
+            const int src = io + 1 + q;
+            e = nd.U[src]; x = T.UA[src]; y = T.UB[src]; ia = T.ia[src]; ib = T.ib[src];
+        } else {
+            e = C.nu[q - m0];
+            const int2 ab = bond_ends(g, e);
+            x = ab.x; y = ab.y; ia = -1; ib = -1;
+        }
+        if (ia < 0 && x == cb) ia = vn;               // the vertex the child brought in
+        if (ib < 0 && y == cb) ib = vn;
+        C.e[q] = e; C.ia[q] = ia; C.ib[q] = ib;
+        C.o[q] = ia < 0 ? x : (ib < 0 ? y : -1);
+    }
+    __syncwarp();
+    const bool v0 = lane < n, v1 = lane + 32 < n;
+    const int o0 = v0 ? C.o[lane] : -2 - lane, o1 = v1 ? C.o[lane + 32] : -2 - lane;
+    const uint64_t inside = (uint64_t)__ballot_sync(0xffffffffu, o0 == -1) |
+                            ((uint64_t)__ballot_sync(0xffffffffu, v1 && o1 == -1) << 32);
+    const uint32_t match0 = __match_any_sync(0xffffffffu, o0);
+    for (int i0 = 0; i0 < n; i0 += 32) {
         const int i = i0 + lane;
-        bool emit = false;
-        int np = 0, d0 = -1, d1 = -1;
-        Child c{-1, -1, -1, 0u, 0};
-        const bool mine = i < nU && ((want >> i) & 1);
+        const bool mine = i < n;
+        int b2 = -1;
+        uint32_t dm2 = 0;
+        uint64_t close = 0;
         if (mine) {
-            c = make_child(T, i, node_dmask);
-            emit = c.dang == 0;
-            if (c.dang <= 2) {
-                for (uint32_t m = c.dmask; m; m &= m - 1) {
-                    const int v = nd.vv[__ffs(m) - 1];
-                    if (d0 < 0) d0 = v; else d1 = v;
+            const int ia = C.ia[i], ib = C.ib[i];
+            b2 = i0 ? o1 : o0;
+            dm2 = cdm & ~((ia >= 0 ? 1u << ia : 0u) | (ib >= 0 ? 1u << ib : 0u));
+        }
+        const int dang = __popc(dm2) + (b2 >= 0 ? 1 : 0);
+        if (mine && dang <= 2) {
+            close = inside;
+            if (b2 >= 0) {
+                uint64_t twin = i0 ? 0u : match0;
+                if (n > 32) {
+                    twin = 0;
+                    for (int q = i + 1; q < n; ++q) twin |= (uint64_t)(C.o[q] == b2) << q;
                 }
-                if (c.b >= 0) { if (d0 < 0) d0 = c.b; else d1 = c.b; }
-                for (int j = i + 1; j < nU; ++j) {
-                    const int oj = T.outside(j);
-                    if (oj != -1 && oj != c.b) continue;
-                    const int x = T.UA[j], y = T.UB[j];
-                    if ((d0 >= 0 && d0 != x && d0 != y) || (d1 >= 0 && d1 != x && d1 != y)) continue;
-                    ++np;
-                }
+                close = twin;                         // the new vertex has degree one: V[j] must touch it
             }
+            close &= i < 63 ? ~0ull << (i + 1) : 0ull;
         }
-        const unsigned em = __ballot_sync(0xffffffffu, emit), pm = __ballot_sync(0xffffffffu, np > 0);
-        emask |= (uint64_t)em << i0;
-        pmask |= (uint64_t)pm << i0;
-        int incl = np;
+        for (uint32_t m = cdm; m; m &= m - 1) {       // candidates at each degree-one vertex of the child
+            const int k = __ffs(m) - 1;
+            const uint64_t at = (uint64_t)__ballot_sync(0xffffffffu, v0 && (C.ia[lane] == k || C.ib[lane] == k)) |
+                                ((uint64_t)__ballot_sync(0xffffffffu, v1 && (C.ia[lane + 32] == k || C.ib[lane + 32] == k)) << 32);
+            if ((dm2 >> k) & 1) close &= at;
+        }
+        const bool emit = mine && dang == 0;
+        const unsigned em = __ballot_sync(0xffffffffu, emit);
+        const int np = __popcll((long long)close);
+        if (WRITE) {
+            int incl = np;
 #pragma unroll
-        for (int off = 1; off < 32; off <<= 1) {
-            const int z = __shfl_up_sync(0xffffffffu, incl, off);
-            if (lane >= off) incl += z;
+            for (int off = 1; off < 32; off <<= 1) {
+                const int z = __shfl_up_sync(0xffffffffu, incl, off);
+                if (lane >= off) incl += z;
+            }
+            const int ec = nd.U[io];
+            if (emit) write_child_cluster(out, slotA + nA + __popc(em & lt), nd, ec, C.e[i], -1, cb, b2);
+            int64_t slot = slotB + nB + (incl - np);
+            for (uint64_t m = close; m; m &= m - 1)
+                write_child_cluster(out, slot++, nd, ec, C.e[i], C.e[__ffsll((long long)m) - 1], cb, b2);
+            nB += __shfl_sync(0xffffffffu, incl, 31);
+        } else {
+            nB += __reduce_add_sync(0xffffffffu, np);
         }
-        if (pass == kEmit && mine) {
-            const int ei = nd.U[i];
-            if (emit) write_child_cluster(out, ebase + n_emit + __popc(em & lt), nd, ei, -1, c.b);
-            int64_t slot = pbase + n_pair + (incl - np);
-            if (np > 0)
-                for (int j = i + 1; j < nU; ++j) {
-                    const int oj = T.outside(j);
-                    if (oj != -1 && oj != c.b) continue;
-                    const int x = T.UA[j], y = T.UB[j];
-                    if ((d0 >= 0 && d0 != x && d0 != y) || (d1 >= 0 && d1 != x && d1 != y)) continue;
-                    write_child_cluster(out, slot++, nd, ei, nd.U[j], c.b);
-                }
-        }
-        n_emit += __popc(em);
-        n_pair += __shfl_sync(0xffffffffu, incl, 31);
+        nA += __popc(em);
     }
-    if (pass == kPairCount && lane == 0) {
-        A.counts[(int64_t)(t + 1) * A.cap + u] = n_emit;
-        A.counts[(int64_t)(t + 2) * A.cap + u] = n_pair;
-        A.emask[u] = emask;
-        A.gmask[u] = pmask;
-    }
+    __syncwarp();
 }
 
 // The block's chunk of the node range [r0, r1).  kChildren writes the
 // children from arena slot next + cbase_chunk on (cbase_chunk: the children of
 // the chunks before this one).
-// With FUSE, nodes of size K - 2 (LOOP mode) are closing nodes (pair_node).
+// With FUSE (LOOP mode, K >= 4) the tables have the three rows of the closing
+// step, and nodes of size K - 3 close their children themselves.
 // One instance per pass keeps each kernel's code small enough for the
 // instruction cache.
 template <int PASS, bool FUSE>
@@ -690,12 +737,15 @@ __device__ void expand_chunk(const GeomView &g, const Arena &A, int64_t r0, int6
     __shared__ uint64_t sh_tmask[kExpandWarps][kNodeV];
     __shared__ int32_t sh_tw[kExpandWarps][kNodeU];
     __shared__ int32_t sh_stage[kExpandWarps][32 * kStageWords];
+    __shared__ int32_t sh_close[kExpandWarps][(pass == kClose || (pass == kEmit && fuse)) ? 4 * kNodeU + kMaxNew : 1];
     __shared__ int64_t wsum[kExpandWarps];
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const unsigned lt = (1u << lane) - 1u;
     Node &nd = sh_node[w];
     const NodeTabs T{sh_a[w], sh_b[w], sh_ia[w], sh_ib[w], sh_tmask[w], sh_tw[w]};
     int32_t *stage = sh_stage[w];
+    const CloseTabs C{sh_close[w], sh_close[w] + kNodeU, sh_close[w] + 2 * kNodeU, sh_close[w] + 3 * kNodeU,
+                      sh_close[w] + 4 * kNodeU};
     // the counting and children passes take contiguous chunks (the child
     // offsets are scanned per chunk); the others stride over the whole range,
     // so the costly nodes of the deepest level spread over every block
@@ -710,9 +760,10 @@ __device__ void expand_chunk(const GeomView &g, const Arena &A, int64_t r0, int6
         uint64_t want = ~0ull;
         if (pass == kChildren) want = __ldcg(reinterpret_cast<const unsigned long long *>(A.gmask + u));
         else if (pass == kEmit) want = __ldcg(reinterpret_cast<const unsigned long long *>(A.emask + u));
-        if (pass == kEmit && fuse && __ldcg(&A.nodes[u].t) == K - 2)   // a closing node: lanes with a closing bond too
-            want |= __ldcg(reinterpret_cast<const unsigned long long *>(A.gmask + u));
-        if (want == 0) continue;
+        uint64_t closes = 0;                             // children with a cluster of size K - 1 or K below them
+        if (pass == kEmit && fuse && __ldcg(&A.nodes[u].t) == K - 3)
+            closes = __ldcg(reinterpret_cast<const unsigned long long *>(A.gmask + u));
+        if ((want | closes) == 0) continue;
         // L2 loads: these nodes were written by other blocks
         const int32_t *src = reinterpret_cast<const int32_t *>(A.nodes + u);
         for (int q = lane; q < kNodeWords; q += 32) reinterpret_cast<int32_t *>(&nd)[q] = __ldcg(src + q);
@@ -730,13 +781,8 @@ __device__ void expand_chunk(const GeomView &g, const Arena &A, int64_t r0, int6
         }
         const uint32_t dmask = __ballot_sync(0xffffffffu, lane < vn && nd.vd[lane] == 1);
         __syncwarp();
-        if (fuse && t == K - 2) {
-            pair_node<PASS>(A, nd, u, T, dmask, want, out);
-            __syncwarp();
-            continue;
-        }
-        const bool closing_children = pass == kCount && fuse && t + 1 == K - 2;
-        if (pass == kCount) {
+        constexpr bool closing_children = pass == kClose;
+        if (pass == kCount || pass == kClose) {
             // the candidates at each vertex of the node
             for (int k = 0; k < vn; ++k) {
                 const unsigned m0 = __ballot_sync(0xffffffffu, lane < nU && (T.ia[lane] == k || T.ib[lane] == k));
@@ -766,7 +812,12 @@ __device__ void expand_chunk(const GeomView &g, const Arena &A, int64_t r0, int6
         }
         int n_child = 0, n_emit = 0;
         const int64_t cbase = (pass == kChildren) ? next + cbase_chunk + __ldcg(A.child_off + u) : 0;
-        const int64_t ebase = (pass == kEmit) ? A.base[(int64_t)(t + 1) * A.cap + u] : 0;
+        const int64_t own_row = fuse ? 0 : (int64_t)(t + 1) * A.cap;
+        const int64_t ebase = (pass == kEmit) ? A.base[own_row + u] : 0;
+        const bool closer = pass == kClose || (pass == kEmit && closes != 0);
+        const int64_t abase = (pass == kEmit && closer) ? A.base[A.cap + u] : 0;
+        const int64_t bbase = (pass == kEmit && closer) ? A.base[2 * A.cap + u] : 0;
+        int nA = 0, nB = 0;
         uint64_t gmask = 0, emask = 0;
         for (int i0 = 0; i0 < nU; i0 += 32) {
             const int i = i0 + lane;
@@ -774,7 +825,7 @@ __device__ void expand_chunk(const GeomView &g, const Arena &A, int64_t r0, int6
             int32_t NU[kMaxNew], NB[kMaxNew];
             int nn = 0;
             Child c{-1, -1, -1, 0u, 0};
-            const bool mine = i < nU && ((want >> i) & 1);
+            const bool mine = i < nU && (((want | closes) >> i) & 1);
             if (mine) {
                 c = make_child(T, i, dmask);
                 const int e = nd.U[i];
@@ -783,10 +834,12 @@ __device__ void expand_chunk(const GeomView &g, const Arena &A, int64_t r0, int6
                     grow = true;
                     if (c.b >= 0) nn = new_candidates(g, c.b, e, anchor, nd.vv, vn, NU, NB, &A.ctl->cand_overflow);
                 } else if (pass == kEmit) {
-                    emit = true;
+                    emit = (want >> i) & 1;
+                    grow = (closes >> i) & 1;
+                    if (grow && c.b >= 0) nn = new_candidates(g, c.b, e, anchor, nd.vv, vn, NU, NB, &A.ctl->cand_overflow);
                 } else {
                     emit = valid_set(mode, c.dang);
-                    if (pass == kCount && may_grow(mode, t + 1, K, c.dang)) {
+                    if ((pass == kCount || pass == kClose) && may_grow(mode, t + 1, K, c.dang)) {
                         if (c.b >= 0) nn = new_candidates(g, c.b, e, anchor, nd.vv, vn, NU, NB, &A.ctl->cand_overflow);
                         grow = mode == PNE_MODE_ALL || repairable_child(T, c, i, nn, nU);
                         if (closing_children && grow) grow = closable2(T, c, i, nn, NB, nU);
@@ -848,14 +901,38 @@ __device__ void expand_chunk(const GeomView &g, const Arena &A, int64_t r0, int6
                 __syncwarp();
             }
             if (pass == kEmit && emit)
-                write_child_cluster(out, ebase + n_emit + __popc(em & lt), nd, nd.U[i], -1, c.b);
+                write_child_cluster(out, ebase + n_emit + __popc(em & lt), nd, nd.U[i], -1, -1, c.b, -1);
+            if constexpr (pass == kClose || (pass == kEmit && fuse)) {
+                // the children that may still close, one after another
+                const uint32_t cdm = c.dmask | (c.b >= 0 ? 1u << vn : 0u);
+                unsigned done = 0;
+                for (unsigned rem = closer ? gm : 0u; rem; rem &= rem - 1) {
+                    const int o = __ffs(rem) - 1;
+                    int nno = __shfl_sync(0xffffffffu, nn, o);
+                    const int io = i0 + o;
+                    if (lane == o)
+                        for (int q = 0; q < nn; ++q) C.nu[q] = NU[q];
+                    __syncwarp();
+                    if (nU - io - 1 + nno > kNodeU) {
+                        if (lane == 0) atomicExch(&A.ctl->cand_overflow, 1);
+                        nno = kNodeU - (nU - io - 1);
+                    }
+                    const int a0 = nA, b0 = nB;
+                    close_child<pass == kEmit>(g, nd, T, C, io, __shfl_sync(0xffffffffu, c.b, o),
+                                               __shfl_sync(0xffffffffu, cdm, o), nno, abase, bbase, nA, nB, out);
+                    if (nA != a0 || nB != b0) done |= 1u << o;
+                }
+                if (pass == kClose) gmask = (gmask & ~((uint64_t)gm << i0)) | ((uint64_t)done << i0);
+            }
             n_child += __popc(gm);
             n_emit += __popc(em);
         }
-        if ((pass == kCount || pass == kEmitCount) && lane == 0) {
-            A.counts[(int64_t)(t + 1) * A.cap + u] = n_emit;
+        if ((pass == kCount || pass == kEmitCount || pass == kClose) && lane == 0) {
+            A.counts[own_row + u] = n_emit;
             A.emask[u] = emask;
-            if (pass == kCount) { A.child_cnt[u] = n_child; A.gmask[u] = gmask; }
+            if (pass == kCount) A.child_cnt[u] = n_child;
+            if (pass != kEmitCount) A.gmask[u] = gmask;
+            if (pass == kClose) { A.counts[A.cap + u] = nA; A.counts[2 * A.cap + u] = nB; }
         }
         __syncwarp();
     }
@@ -868,7 +945,7 @@ __device__ void expand_chunk(const GeomView &g, const Arena &A, int64_t r0, int6
     __syncthreads();                                   // the shared node buffers are reused by the caller
 }
 
-// kCount / kEmitCount / kPairCount of level lo == hi, or kEmit over levels lo..hi
+// kCount / kEmitCount / kClose of level lo == hi, or kEmit over levels lo..hi
 template <int PASS, bool FUSE>
 __global__ void __launch_bounds__(32 * kExpandWarps, 6)
 expand_kernel(GeomView g, Arena A, int lo_level, int hi_level, int K, int mode, Emit out)
@@ -1182,10 +1259,13 @@ pne_status scan_i32_to(pne_ctx *ctx, const int32_t *src, int64_t *dst, int64_t n
 // row starts are gathered on the device and their copy to pinned memory is
 // queued, together with `extra_bytes` from `extra_dev` (a multiple of 8);
 // *h_out receives the pinned words (rows + 1 starts, then the extra bytes).
+// With close_lv (the level bounds of a search with the closing step at order
+// rows - 1) the table has three rows instead, see close_starts_kernel.
 pne_status scan_counts_queue(pne_ctx *ctx, const int32_t *d_counts, int rows, int64_t cols, DevBuf &base,
-                             cudaStream_t s, int64_t **h_out, const void *extra_dev = nullptr, size_t extra_bytes = 0)
+                             cudaStream_t s, int64_t **h_out, const void *extra_dev = nullptr, size_t extra_bytes = 0,
+                             const int64_t *close_lv = nullptr)
 {
-    const int64_t n = (int64_t)rows * cols;
+    const int64_t n = (int64_t)(close_lv ? 3 : rows) * cols;
     pne_status st = dev_alloc(ctx, base, (size_t)(std::max<int64_t>(n, 1) + rows + 3) * 8, s);
     if (st) return st;
     int64_t *b = (int64_t *)base.ptr;
@@ -1193,7 +1273,8 @@ pne_status scan_counts_queue(pne_ctx *ctx, const int32_t *d_counts, int rows, in
     int64_t *tot = starts + rows + 1;                       // [1]
     // exclusive scan; its total lands in tot
     if ((st = scan_i32_to(ctx, d_counts, b, n, tot, s))) return st;
-    row_starts_kernel<<<(rows + 1 + 127) / 128, 128, 0, s>>>(b, rows, cols, n, starts, tot);
+    if (close_lv) close_starts_kernel<<<1, 64, 0, s>>>(b, cols, close_lv, rows - 1, starts, tot);
+    else row_starts_kernel<<<(rows + 1 + 127) / 128, 128, 0, s>>>(b, rows, cols, n, starts, tot);
     PNE_LAUNCH_CHECK(ctx);
     const size_t words = (size_t)(rows + 1) + extra_bytes / 8;
     int64_t *h = pinned_i64(ctx, words);
@@ -1208,10 +1289,10 @@ pne_status scan_counts_queue(pne_ctx *ctx, const int32_t *d_counts, int rows, in
 // bytes into extra_host.
 pne_status scan_counts(pne_ctx *ctx, const int32_t *d_counts, int rows, int64_t cols, DevBuf &base,
                        std::vector<int64_t> &row_tot, cudaStream_t s, const void *extra_dev = nullptr,
-                       size_t extra_bytes = 0, void *extra_host = nullptr)
+                       size_t extra_bytes = 0, void *extra_host = nullptr, const int64_t *close_lv = nullptr)
 {
     int64_t *h = nullptr;
-    pne_status st = scan_counts_queue(ctx, d_counts, rows, cols, base, s, &h, extra_dev, extra_bytes);
+    pne_status st = scan_counts_queue(ctx, d_counts, rows, cols, base, s, &h, extra_dev, extra_bytes, close_lv);
     if (st) return st;
     {
         HostScope hw__(ctx, "sync_counts");
@@ -1233,7 +1314,7 @@ void launch_expand(int pass, bool fuse, int G, cudaStream_t s, const GeomView &g
         else expand_kernel<kCount, false><<<G, T, 0, s>>>(gv, A, lo, hi, K, mode, o);
         break;
     case kEmitCount: expand_kernel<kEmitCount, false><<<G, T, 0, s>>>(gv, A, lo, hi, K, mode, o); break;
-    case kPairCount: expand_kernel<kPairCount, true><<<G, T, 0, s>>>(gv, A, lo, hi, K, mode, o); break;
+    case kClose: expand_kernel<kClose, true><<<G, T, 0, s>>>(gv, A, lo, hi, K, mode, o); break;
     default:
         if (fuse) expand_kernel<kEmit, true><<<G, T, 0, s>>>(gv, A, lo, hi, K, mode, o);
         else expand_kernel<kEmit, false><<<G, T, 0, s>>>(gv, A, lo, hi, K, mode, o);
@@ -1258,12 +1339,13 @@ pne_status enumerate_clusters(pne_ctx *ctx, const Geometry &g, int K, int mode, 
     }
     if ((kPrefixMax + 1) * (maxdeg - 1) > kNodeU) { set_error(ctx, PNE_EINVAL, "site degree too large"); return PNE_EINVAL; }
     GeomView gv{g.d_bond_site, g.d_site_ptr, g.d_site_bonds, g.d_site_nbr};
-    // prefix levels 1..D are expanded breadth-first; the last one closes both
-    // remaining sizes (LOOP mode, D == K - 2), only emits (D == K - 1) or is
-    // searched depth-first (K - 1 > kPrefixMax)
-    const bool fuse = mode == PNE_MODE_LOOP && K >= 3 && K - 2 <= kPrefixMax;
-    const int D = fuse ? K - 2 : ((K <= 1) ? 1 : std::min(kPrefixMax, K - 1));
-    const int final_kind = fuse ? 3 : ((K <= 1) ? 0 : (D == K - 1 ? 1 : 2));
+    // prefix levels 1..D are expanded breadth-first; the last one closes the
+    // three remaining sizes (LOOP mode, D == K - 3), only emits (D == K - 1) or
+    // is searched depth-first (K - 1 > kPrefixMax)
+    bool fuse = mode == PNE_MODE_LOOP && K >= 4 && K - 3 <= kPrefixMax;
+    auto levels = [&] { return fuse ? K - 3 : ((K <= 1) ? 1 : std::min(kPrefixMax, K - 1)); };
+    int D = levels();
+    int final_kind = fuse ? 3 : ((K <= 1) ? 0 : (D == K - 1 ? 1 : 2));
     const bool small = (K <= 12 && umax_need <= 64);
     // chunks of the blocked passes: one wave of resident blocks (the occupancy
     // is queried once per context)
@@ -1282,6 +1364,13 @@ pne_status enumerate_clusters(pne_ctx *ctx, const Geometry &g, int K, int mode, 
         auto it = ctx->arena_hint.find(hint_key);
         if (it != ctx->arena_hint.end()) cap = it->second;
     }
+    auto no_closing = [&] {           // the levels do not fit the largest arena: depth-first below one that does
+        fuse = false;
+        D = levels();
+        final_kind = D == K - 1 ? 1 : 2;
+        cap = INT64_MAX;
+    };
+    if (cap < 0) no_closing();        // known from the last search of this geometry
     const int64_t cap_max = ctx->arena_max > 0 ? std::max<int64_t>(ctx->arena_max, Mc) : kNodeCap;
     cap = std::min(cap_max, std::max<int64_t>(cap, Mc));
     Emit none{nullptr, nullptr, nullptr, rec.width, rec.vwidth};
@@ -1307,7 +1396,8 @@ pne_status enumerate_clusters(pne_ctx *ctx, const Geometry &g, int K, int mode, 
         if ((st = dev_alloc(ctx, nodes, sizeof(Node) * (size_t)cap, s))) return st;
         const size_t tab_bytes = sizeof(Readback) + (size_t)cap * 4 + (size_t)cap * 24 + (size_t)G * 8 + 64;
         if ((st = dev_alloc(ctx, tables, tab_bytes, s))) return st;
-        if ((st = dev_alloc(ctx, counts, (size_t)(K + 1) * cap * 4, s))) return st;
+        const int rows = fuse ? 3 : K + 1;
+        if ((st = dev_alloc(ctx, counts, (size_t)rows * cap * 4, s))) return st;
         char *tb = (char *)tables.ptr;
         A.nodes = (Node *)nodes.ptr;
         A.cap = cap;
@@ -1320,7 +1410,7 @@ pne_status enumerate_clusters(pne_ctx *ctx, const Geometry &g, int K, int mode, 
         A.child_cnt = (int32_t *)(A.emask + cap);
         A.counts = (int32_t *)counts.ptr;
         A.base = nullptr;
-        PNE_CUDA_TRY(ctx, cudaMemsetAsync(counts.ptr, 0, (size_t)(K + 1) * cap * 4, s));
+        PNE_CUDA_TRY(ctx, cudaMemsetAsync(counts.ptr, 0, (size_t)rows * cap * 4, s));
         arena_init_kernel<<<1, 32, 0, s>>>(A, Mc);
         PNE_LAUNCH_CHECK(ctx);
         {
@@ -1343,14 +1433,16 @@ pne_status enumerate_clusters(pne_ctx *ctx, const Geometry &g, int K, int mode, 
         }
         if (final_kind == 1 || final_kind == 3) {
             ProfScope ps__(ctx, s, "enum_close_count");
-            launch_expand(final_kind == 3 ? kPairCount : kEmitCount, final_kind == 3, G, s, gv, A, D, D, K, mode, none);
+            launch_expand(final_kind == 3 ? kClose : kEmitCount, final_kind == 3, G, s, gv, A, D, D, K, mode, none);
         } else if (final_kind == 2) {
             dfs(A, D, 0, none);
         }
         PNE_LAUNCH_CHECK(ctx);
         // one (size, node) table over the arena; the same round trip brings the
         // level bounds and the stop record
-        if ((st = scan_counts(ctx, A.counts, K + 1, cap, base, per_size, s, A.lv, sizeof(Readback), &hb))) return st;
+        if ((st = scan_counts(ctx, A.counts, K + 1, cap, base, per_size, s, A.lv, sizeof(Readback), &hb,
+                              fuse ? A.lv : nullptr)))
+            return st;
         if (hb.ctl.cand_overflow) {
             set_error(ctx, PNE_EOVERFLOW, "candidate list overflow in the cluster search");
             return PNE_EOVERFLOW;
@@ -1359,6 +1451,12 @@ pne_status enumerate_clusters(pne_ctx *ctx, const Geometry &g, int K, int mode, 
         if (cap < cap_max) {
             // the tree outgrew the arena: grow it and search again
             cap = std::min(cap_max, std::max(4 * cap, 2 * hb.ctl.need));
+            dev_free(ctx, nodes, s); dev_free(ctx, tables, s); dev_free(ctx, counts, s); dev_free(ctx, base, s);
+            continue;
+        }
+        if (fuse) {
+            no_closing();
+            cap = cap_max;
             dev_free(ctx, nodes, s); dev_free(ctx, tables, s); dev_free(ctx, counts, s); dev_free(ctx, base, s);
             continue;
         }
@@ -1375,7 +1473,8 @@ pne_status enumerate_clusters(pne_ctx *ctx, const Geometry &g, int K, int mode, 
         const int last = hb.ctl.stop ? hb.ctl.stop : D;
         const int64_t used = ((hb.lv[last] + 1023) / 1024) * 1024;
         std::lock_guard<std::mutex> lk(ctx->cache_mu);
-        ctx->arena_hint[hint_key] = std::min(cap_max, std::max<int64_t>(used, 1024));
+        const bool closing_failed = !fuse && mode == PNE_MODE_LOOP && K >= 4 && K - 3 <= kPrefixMax;
+        ctx->arena_hint[hint_key] = closing_failed ? -1 : hb.ctl.stop ? cap_max : std::max<int64_t>(used, 1024);
     }
     uint64_t n_cl = 0;
     rec.size_start.assign(K + 2, 0);
@@ -1398,7 +1497,7 @@ pne_status enumerate_clusters(pne_ctx *ctx, const Geometry &g, int K, int mode, 
     PNE_LAUNCH_CHECK(ctx);
     if (last_bfs >= 1) {
         ProfScope ps__(ctx, s, "enum_emit");
-        launch_expand(kEmit, final_kind == 3 && dfs_level == 0, G, s, gv, A, 1, last_bfs, K, mode, out);
+        launch_expand(kEmit, final_kind == 3, G, s, gv, A, 1, last_bfs, K, mode, out);
     }
     PNE_LAUNCH_CHECK(ctx);
     if (dfs_level) dfs(A, dfs_level, 1, out);
