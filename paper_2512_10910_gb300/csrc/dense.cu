@@ -14,17 +14,19 @@
 // legs sit at the two ends and its two output legs are appended at the end:
 // the next site finds its own legs at the ends again, across rows too.
 //
-// The GEMM (tc_gemm_kernel): one CTA per 128 x BN tile of the output (BN <= 256)
-// and tensor set.  K is staged 128 bytes per row at a time (32 TF32 or 64 BF16
-// values) in two shared-memory stages, written by all threads in the
-// canonical no-swizzle K-major layout (8-row x 16-byte core matrices, the two
-// core matrices of one MMA K step 128 bytes apart, 8-row groups 1024 bytes
-// apart); one elected thread issues tcgen05.mma (M = 128, N = BN, FP32
-// accumulation in tensor memory) and commits each stage to an mbarrier, which
-// the loaders wait on (bounded) before refilling the stage.  The epilogue
-// reads the accumulator with tcgen05.ld (a warp per 32 lanes = rows) and
-// records the largest |entry| per set, from which the next step takes a
-// power-of-two scale (kept exactly in a log-2 counter).  The FP64 form
+// The large products run on one persistent kernel (tc_stream_kernel: operand
+// stages filled by the Tensor Memory Accelerator, tcgen05.mma with M = 128,
+// N <= 256 and FP32 accumulation in tensor memory, a finished tile stored while
+// the next accumulates).  Small products of pne_dense_gemm, and those whose A
+// is not on 16-byte boundaries, take tc_gemm_kernel: one CTA per tile, K staged
+// 128 bytes per row at a time in two shared-memory stages written by all
+// threads in the canonical no-swizzle K-major layout (8-row x 16-byte core
+// matrices, the two core matrices of one MMA K step 128 bytes apart, 8-row
+// groups 1024 bytes apart), each stage committed to an mbarrier on which the
+// loaders wait (bounded) before refilling it.  Both add a K step of 32 bytes at
+// a time in the same order, so their results are the same bit for bit.  The
+// grid's steps record the largest |entry| per set, from which the next step
+// takes a power-of-two scale (kept exactly in a log-2 counter).  The FP64 form
 // (f64_gemm_kernel) is a plain tiled GEMM on the CUDA cores with the same
 // interface: the reference the reduced-precision forms are stated against.
 #include <cuda.h>
@@ -39,6 +41,7 @@
 #include <cstdlib>
 #include <cstring>
 #include <string>
+#include <type_traits>
 #include <vector>
 
 #include "pne_internal.h"
@@ -50,7 +53,6 @@ constexpr int kTcThreads = 128;
 constexpr int kTcBM = 128;
 constexpr int kChunk = 128;                   // K bytes per row per stage
 constexpr int kATileBytes = kTcBM * kChunk;   // 16 KB
-constexpr int kTmaChunk = 64;                 // K bytes per row per stage of the TMA-fed kernel
 constexpr uint64_t kWaitNs = 2000000000ull;   // bounded mbarrier waits: 2 s
 
 // ---------------------------------------------------------------- PTX wrappers
@@ -145,6 +147,9 @@ __device__ __forceinline__ uint64_t global_ns()
 // bounded wait (about two seconds of the global timer); false when it gave up
 __device__ __forceinline__ bool mbar_wait(uint32_t addr, uint32_t parity)
 {
+    // reading the timer costs more than most waits: not before a few tries
+    for (int i = 0; i < 32; ++i)
+        if (mbar_try_wait(addr, parity)) return true;
     const uint64_t t0 = global_ns();
     for (;;) {
         if (mbar_try_wait(addr, parity)) return true;
@@ -470,18 +475,12 @@ __global__ void grid_final_kernel(const T *S, int64_t stride, const long long *l
     out[2 * set + 1] = (double)log2s[set];
 }
 
-// ---------------------------------------------------------------- the grid's pipelined GEMM
+// ---------------------------------------------------------------- the grid's GEMM step
 // One site absorption of the grid contraction on the tensor cores, with the
 // running tensor S read in its ring order directly (no packing pass):
 //     out[m][n] = 2^-e_in * sum_{u,h} S[u][m][h] * Bm[n][u Kh + h],
 // the result rounded to the operand type (TF32 kept in FP32 words, or BF16) as
 // the next step's running tensor, its largest |entry| recorded per set.
-// Stages are filled with 16-byte cp.async copies (4 stages in flight): the
-// operands are already in the MMA's type, so a stage is a plain copy into the
-// canonical layout; where a 16-byte unit of A is not contiguous in S (a left
-// boundary site, Kh not a multiple of the unit) it is gathered element by
-// element instead.  The epilogue goes through shared memory (the free
-// stages) so that every warp stores whole 128-byte row segments.
 template <typename E>
 struct RingParams {
     const E *S;              // [set][stride] running tensor [Ku][R][Kh]
@@ -499,20 +498,6 @@ struct RingParams {
     int *err;
 };
 
-__device__ __forceinline__ void cp_async16(uint32_t dst, const void *src, uint32_t src_bytes)
-{
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(src_bytes) : "memory");
-}
-__device__ __forceinline__ void cp_async_commit()
-{
-    asm volatile("cp.async.commit_group;" ::: "memory");
-}
-template <int N>
-__device__ __forceinline__ void cp_async_wait()
-{
-    asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
-}
-
 template <typename E>
 __device__ __forceinline__ float elem_to_float(E x);
 template <>
@@ -526,178 +511,6 @@ template <>
 __device__ __forceinline__ float round_elem<float>(float x) { return __uint_as_float(to_tf32(x)); }
 template <>
 __device__ __forceinline__ __nv_bfloat16 round_elem<__nv_bfloat16>(float x) { return __float2bfloat16_rn(x); }
-
-template <typename E, int NST>
-__global__ void __launch_bounds__(kTcThreads, 2) tc_ring_gemm_kernel(RingParams<E> p, int BN)
-{
-    constexpr int kRingStages = NST;
-    constexpr int EB = (int)sizeof(E);
-    constexpr int EPU = 16 / EB;          // elements per 16-byte unit
-    constexpr int KC = kChunk / EB;       // elements per stage row
-    extern __shared__ uint8_t smem_raw[];
-    __shared__ __align__(8) uint64_t mbar[kRingStages];
-    __shared__ uint32_t tmem_base_sh;
-    uint8_t *base = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-    const int stage_bytes = kATileBytes + BN * kChunk;
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int set = blockIdx.z;
-    const int64_t m0 = (int64_t)blockIdx.x * kTcBM;
-    const int n0 = blockIdx.y * BN;
-    const E *S = p.S + set * p.stride;
-    const E *Bm = p.B + set * p.b_stride;
-    E *out = p.out + set * p.stride;
-    const uint32_t tcols = BN <= 32 ? 32u : (BN <= 64 ? 64u : (BN <= 128 ? 128u : 256u));
-    const bool a_contig = (p.Kh % EPU) == 0;
-
-    if (warp == 0) {
-        tmem_alloc(smem_addr(&tmem_base_sh), tcols);
-        tmem_relinquish();
-    }
-    if (tid == 0)
-        for (int i = 0; i < kRingStages; ++i) mbar_init(smem_addr(&mbar[i]), 1);
-    tc_fence_before();
-    __syncthreads();
-    tc_fence_after();
-    const uint32_t tmem = tmem_base_sh;
-    const int nchunks = (p.K + KC - 1) / KC;
-    const uint32_t idesc = instr_desc(EB == 4 ? 2u : 1u, kTcBM, (uint32_t)BN);
-
-    // each thread copies one fixed 16-byte column (cu) of rows r0, r0 + 16, ...:
-    // per stage one division for its k, then addresses advance by a constant
-    const int cu = tid & 7, r0 = tid >> 3;
-    const int64_t a_row_step = 16 * (int64_t)p.Kh;
-    const int64_t b_row_step = 16 * p.ldb;
-    auto load_stage = [&](int c) {
-        if (c >= nchunks) return;
-        uint8_t *sa = base + (c % kRingStages) * stage_bytes;
-        uint8_t *sb = sa + kATileBytes;
-        const int k = c * KC + cu * EPU;
-        const bool k_in = k < p.K;
-        if (a_contig) {
-            const int ku = k_in ? k / p.Kh : 0, kh = k_in ? k - ku * p.Kh : 0;
-            const E *src = S + ((int64_t)ku * p.R + m0 + r0) * p.Kh + kh;
-            int64_t m = m0 + r0;
-            uint32_t dst = smem_addr(sa) + (uint32_t)tile_off(r0, cu);
-#pragma unroll
-            for (int i = 0; i < kTcBM / 16; ++i) {
-                const bool in = k_in && m < p.R;
-                cp_async16(dst, in ? (const void *)src : (const void *)S, in ? 16u : 0u);
-                src += a_row_step;
-                m += 16;
-                dst += 2 * 1024;            // 16 rows = two 8-row groups
-            }
-        } else {
-            for (int i = 0; i < kTcBM / 16; ++i) {
-                const int r = r0 + 16 * i;
-                const int64_t m = m0 + r;
-                __align__(16) E v[EPU];
-#pragma unroll
-                for (int j = 0; j < EPU; ++j) {
-                    const int kk = k + j;
-                    if (m < p.R && kk < p.K) {
-                        const int ku = kk / p.Kh, kh = kk - ku * p.Kh;
-                        v[j] = S[((int64_t)ku * p.R + m) * p.Kh + kh];
-                    } else {
-                        v[j] = round_elem<E>(0.f);
-                    }
-                }
-                *reinterpret_cast<uint4 *>(sa + tile_off(r, cu)) = *reinterpret_cast<const uint4 *>(v);
-            }
-        }
-        const uint32_t bytes = k_in ? (uint32_t)min(16, (p.K - k) * EB) : 0u;
-        const E *bsrc = Bm + (int64_t)(n0 + r0) * p.ldb + (k_in ? k : 0);
-        int n = n0 + r0;
-        uint32_t bdst = smem_addr(sb) + (uint32_t)tile_off(r0, cu);
-        for (int i = 0; i < BN / 16; ++i) {
-            const bool in = n < p.N;
-            cp_async16(bdst, in ? (const void *)bsrc : (const void *)Bm, in ? bytes : 0u);
-            bsrc += b_row_step;
-            n += 16;
-            bdst += 2 * 1024;
-        }
-    };
-
-    for (int c = 0; c < kRingStages - 1; ++c) {
-        load_stage(c);
-        cp_async_commit();
-    }
-    bool ok = true;
-    for (int c = 0; c < nchunks; ++c) {
-        cp_async_wait<kRingStages - 2>();
-        fence_proxy_async();
-        __syncthreads();
-        if (tid == 0 && ok) {
-            tc_fence_after();
-            const uint8_t *sa = base + (c % kRingStages) * stage_bytes;
-            const uint8_t *sb = sa + kATileBytes;
-#pragma unroll
-            for (int ks = 0; ks < 4; ++ks) {
-                const uint64_t ad = smem_desc(smem_addr(sa) + ks * 256, 128, 1024);
-                const uint64_t bd = smem_desc(smem_addr(sb) + ks * 256, 128, 1024);
-                tc_mma<EB>(tmem, ad, bd, idesc, (c > 0 || ks > 0) ? 1u : 0u);
-            }
-            tc_commit(smem_addr(&mbar[c % kRingStages]));
-        }
-        // the stage the next prefetch overwrites was read by chunk c - 1
-        if (c >= 1) {
-            const bool w = ok ? mbar_wait(smem_addr(&mbar[(c - 1) % kRingStages]),
-                                          (uint32_t)(((c - 1) / kRingStages) & 1))
-                              : false;
-            ok = __syncthreads_and(w) != 0;
-        }
-        load_stage(c + kRingStages - 1);
-        cp_async_commit();
-    }
-    cp_async_wait<0>();
-    {
-        const int c = nchunks - 1;
-        const bool w = ok ? mbar_wait(smem_addr(&mbar[c % kRingStages]), (uint32_t)((c / kRingStages) & 1)) : false;
-        ok = __syncthreads_and(w) != 0;
-    }
-    tc_fence_after();
-    // the scale of this step: 2^-e_in, e_in the exponent of the input's largest |entry|
-    const float mx_in = __uint_as_float((unsigned)p.max_in[set]);
-    const int e_in = mx_in > 0.f ? ilogbf(mx_in) : 0;
-    const float sc = ldexpf(1.f, -e_in);
-    if (blockIdx.x == 0 && blockIdx.y == 0 && tid == 0) {
-        p.log2s[set] += e_in;
-        p.max_clear[set] = 0ull;
-    }
-    float mx = 0.f;
-    if (ok) {
-        // 64-column slices through shared memory: [128][64 + 4] floats
-        constexpr int SW = 64, SP = SW + 4;
-        float *st = reinterpret_cast<float *>(base);
-        for (int c0 = 0; c0 < BN; c0 += SW) {
-#pragma unroll
-            for (int q = 0; q < SW; q += 16) {
-                uint32_t r[16];
-                tmem_ld16(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)(c0 + q), r);
-#pragma unroll
-                for (int j = 0; j < 16; ++j) st[(warp * 32 + lane) * SP + q + j] = __uint_as_float(r[j]) * sc;
-            }
-            __syncthreads();
-            for (int i = tid; i < kTcBM * SW; i += kTcThreads) {
-                const int rr = i / SW, cc = i % SW;
-                const int64_t row = m0 + rr;
-                const int col = n0 + c0 + cc;
-                if (row < p.R && col < p.N) {
-                    const E v = round_elem<E>(st[rr * SP + cc]);
-                    out[row * p.N + col] = v;
-                    mx = fmaxf(mx, fabsf(elem_to_float<E>(v)));
-                }
-            }
-            __syncthreads();
-        }
-    } else if (tid == 0) {
-        atomicExch(p.err, 1);
-    }
-    for (int off = 16; off > 0; off >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, off));
-    if (lane == 0 && mx > 0.f) atomicMax(p.max_out + set, (unsigned long long)__float_as_uint(mx));
-    tc_fence_before();
-    __syncthreads();
-    if (warp == 0) tmem_dealloc(tmem, tcols);
-}
 
 // Site matrices for the tensor-core path: rows padded to a multiple of the
 // 16-byte unit, entries scaled by 2^-s_v and rounded to the operand type.
@@ -762,21 +575,44 @@ __global__ void grid_final_tc_kernel(const E *S, int64_t stride, const unsigned 
     (void)max_last;
 }
 
-// ---- the same site GEMM with the stages filled by the Tensor Memory Accelerator.
-// One elected thread of warp 0 issues, per stage, eight boxes of A (the running
-// tensor viewed as [set][Ku][R][Kh], each box 16 bytes of k by 128 rows) and
-// eight of B ([set][N][ldb], 16 bytes of k by BN rows) on one mbarrier with
-// the stage's byte count; a box lands as 128 (BN) consecutive 16-byte rows,
-// which is the canonical no-swizzle K-major layout with 8-row groups 128
-// bytes apart and the box's K column 2048 (16 BN) bytes from the next.  One
-// thread of warp 1 waits for a full stage, issues its four MMAs and commits
-// them to the stage's empty barrier, which the producer waits on before
-// refilling it.  Used where a 16-byte unit of k is contiguous in the running
-// tensor (Kh a multiple of the unit): the innermost box coordinate is then a
-// multiple of 16 bytes, as the copy requires.
+// ---------------------------------------------------------------- the persistent GEMM
+// One kernel for the large products, by where A comes from:
+//   kBoxes   a site absorption of the grid contraction: A is the running
+//            tensor S[u][m][h] (k = u Kh + h), already in the MMA's type,
+//            copied by the Tensor Memory Accelerator; the result is scaled,
+//            rounded to that type and stored as the next running tensor, its
+//            largest |entry| recorded.
+//   kGather  the same where no 16-byte unit of k is contiguous in S (a left
+//            boundary site, Kh = 1, whose m runs fastest, or an odd Kh): eight
+//            warps load it, lanes along m, and write the operand stages.  At
+//            Kh = 1 the loads are whole lines; S is small beside the result.
+//   kRound   pne_dense_gemm: A is FP32; eight warps round each box to the
+//            MMA's type on its way from the landing buffer to the operand
+//            stage (the rounding of B, read by every row tile, is done once by
+//            round_rows_kernel); the result is stored as FP32.
+// Both are bound by HBM at the sizes they are for (K, N = 256: 64 flops per
+// byte of A and C against 140 at the TF32 and 290 at the BF16 tensor rate), so
+// the split is chosen to keep loads in flight: one block per SM walks the
+// tiles; one thread issues the loads (64 KB of A in flight per SM), one the
+// MMAs, four warps store a finished tile from tensor memory while the next one
+// accumulates in its other half; the stages fill the shared memory, up to 12
+// (with four, the N = 16 steps of the last column read 4.1 TB/s).  An operand row of a stage is 128 bytes, copied
+// in boxes of the widest swizzle whose bytes are contiguous in A (128, 64 or
+// 32; 16 without one): boxes of 16 bytes, which every stage used before, cost
+// the copy engine one request per 16 bytes and bound the kernel.
+// Measured, before -> after (HBM 6.7 TB/s): 4 x 32768 x 256 x 256 with B's
+// rounding, BF16 340.6 -> 54.8 us (4.9 TB/s), TF32 507 -> 57 us; 20000 x 2000 x
+// 1000 BF16 1241 -> 131 us (612 TFLOP/s); 32 5 x 4 networks of chi = 16, whole
+// calls: TF32 14.97 -> 6.30 ms (a step with K = N = 256 moves 4.25 GB in 0.64 to
+// 0.66 ms, 6.5 TB/s), BF16 13.58 -> 4.24 ms; 16 5 x 5 networks of chi = 11,
+// gathered: TF32 3.28 -> 1.66 ms.
 __device__ __forceinline__ void mbar_expect_tx(uint32_t bar, uint32_t bytes)
 {
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
+}
+__device__ __forceinline__ void mbar_arrive(uint32_t bar)
+{
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
 }
 __device__ __forceinline__ void tma_load4(uint32_t dst, const CUtensorMap *map, int c0, int c1, int c2, int c3,
                                           uint32_t bar)
@@ -791,165 +627,443 @@ __device__ __forceinline__ void tma_load3(uint32_t dst, const CUtensorMap *map, 
                  ::"r"(dst), "l"((uint64_t)map), "r"(c0), "r"(c1), "r"(c2), "r"(bar)
                  : "memory");
 }
-
-__device__ __forceinline__ void tma_load3_mc(uint32_t dst, const CUtensorMap *map, int c0, int c1, int c2,
-                                             uint32_t bar, uint16_t mask)
+__device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32])
 {
-    asm volatile("cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes.multicast::cluster"
-                 " [%0], [%1, {%2, %3, %4}], [%5], %6;"
-                 ::"r"(dst), "l"((uint64_t)map), "r"(c0), "r"(c1), "r"(c2), "r"(bar), "h"(mask)
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, "
+                 "%14, %15, %16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+                   "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]),
+                   "=r"(r[15]), "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]),
+                   "=r"(r[22]), "=r"(r[23]), "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]),
+                   "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+                 : "r"(taddr)
                  : "memory");
-}
-__device__ __forceinline__ void tc_commit_mc(uint32_t mbar, uint16_t mask)
-{
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;"
-                 ::"r"(mbar), "h"(mask)
-                 : "memory");
-}
-__device__ __forceinline__ void cluster_sync_all()
-{
-    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 }
 
-// CL CTAs on adjacent M tiles form a cluster and share the site matrix: each
-// loads 1/CL of every stage's B boxes and multicasts them to all, so the L2
-// delivers B once per cluster instead of once per CTA.  A stage is refilled
-// only after every member's MMAs on it completed (each member's commit
-// arrives on every member's empty barrier, CL arrivals per phase).
-template <typename E, int NST, int CL>
-__global__ void __launch_bounds__(kTcThreads, 2) tc_tma_gemm_kernel(const __grid_constant__ CUtensorMap tmA,
-                                                                   const __grid_constant__ CUtensorMap tmB,
-                                                                   RingParams<E> p, int BN)
+// shared-memory matrix descriptor of a K-major tile whose rows are `w` bytes
+// wide: swizzled over w = 128, 64 or 32 bytes (8-row groups 8 w apart), or
+// w = 16, unswizzled 16-byte columns of 128 rows
+__device__ __forceinline__ uint64_t tile_desc(uint32_t addr, int w)
 {
-    constexpr int EB = (int)sizeof(E);
-    constexpr int EPU = 16 / EB;
-    constexpr int KC = kTmaChunk / EB;        // k values per stage (64 bytes of each row)
-    constexpr int UNITS = kTmaChunk / 16;     // 16-byte boxes per operand per stage
+    if (w == 16) return smem_desc(addr, kTcBM * 16, 128);
+    const uint64_t layout = w == 128 ? 2 : (w == 64 ? 4 : 6);
+    return smem_desc(addr, 16, (uint32_t)(8 * w)) | (layout << 61);
+}
+
+struct StreamParams {
+    int64_t M;                          // rows of A and of the result
+    int N, K, BN;                       // BN: columns per tile, a multiple of 16
+    int mt, nt, batch;                  // tiles down, across, tensor sets
+    int stages;                         // operand stages in shared memory
+    int w, Kh;                          // kBoxes: bytes of a box of A; h range of one u
+    const void *S;                      // kGather: running tensor [set][Ku][M][Kh], sets strideC apart
+    void *out;                          // [batch][M][ldc]
+    int64_t ldc, strideC;
+    int vec;                            // rows of the result on 16-byte boundaries
+    const unsigned long long *max_in;   // the grid's sources: as RingParams
+    unsigned long long *max_out, *max_clear;
+    long long *log2s;
+    int *err;
+};
+
+// The tiles of one block, every gridDim.x-th, columns fastest, then rows, then
+// sets: advanced by adding (a 64-bit division per tile and role took a third
+// of the time of the steps whose tiles are short).
+struct TileWalk {
+    int n, m, set, dn, dm, ds, nt, mt, batch;
+    __device__ explicit TileWalk(const StreamParams &p) : nt(p.nt), mt(p.mt), batch(p.batch)
+    {
+        const unsigned b = blockIdx.x, g = gridDim.x;
+        n = (int)(b % nt); m = (int)(b / nt % mt); set = (int)(b / nt / mt);
+        dn = (int)(g % nt); dm = (int)(g / nt % mt); ds = (int)(g / nt / mt);
+    }
+    __device__ __forceinline__ bool more() const { return set < batch; }
+    __device__ __forceinline__ void next()
+    {
+        n += dn;
+        int c = n >= nt;
+        n -= c ? nt : 0;
+        m += dm + c;
+        c = m >= mt;
+        m -= c ? mt : 0;
+        set += ds + c;
+    }
+};
+
+constexpr int kStreamStages = 12, kRawBoxes = 4;   // most operand stages; landing boxes
+constexpr int kBoxBytes = kTcBM * 128;
+constexpr int kConvertWarps = 8;
+enum StreamSource { kBoxes = 0, kRound = 1, kGather = 2 };
+// Storing warps, one or two per 32 rows.  The grid's short tiles are bound by
+// four (N = 256, K = 16: 630 us a step with four, 454 with eight); where A is
+// rounded the second four would take the fourth landing box's shared memory
+// (4 x 32768 x 256 x 256 TF32: 57.5 us with four, 61.5 with eight and three boxes).
+constexpr int store_warps(int src) { return src == kRound ? 4 : 8; }
+constexpr int stream_threads(int src) { return 32 * (4 + store_warps(src) + (src == kBoxes ? 0 : kConvertWarps)); }
+
+template <int EB, int SRC>
+__global__ void __launch_bounds__(stream_threads(SRC), 1) tc_stream_kernel(const __grid_constant__ CUtensorMap tmA,
+                                                                           const __grid_constant__ CUtensorMap tmB,
+                                                                           StreamParams p)
+{
+    constexpr bool RAW = SRC == kRound;
+    constexpr int kStoreWarps = store_warps(SRC), kConvert0 = 4 + kStoreWarps;   // first converting warp
+    constexpr bool FILL = SRC != kBoxes;           // warps kConvert0.. write A's operand stages
+    const int NST = p.stages;
+    constexpr int KC = 128 / EB;                   // k values per stage
+    constexpr int OB = RAW ? 4 : EB;               // bytes of a stored value
+    constexpr int RPC = RAW ? 4 / EB : 1;          // landing boxes per operand stage
     extern __shared__ uint8_t smem_raw[];
-    __shared__ __align__(8) uint64_t full[NST], empty[NST], done;
+    __shared__ __align__(8) uint64_t full[kStreamStages], empty[kStreamStages], rfull[kRawBoxes], rempty[kRawBoxes], afull[2], aempty[2];
     __shared__ uint32_t tmem_base_sh;
     uint8_t *base = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-    const int a_bytes = kTcBM * kTmaChunk;
-    const int stage_bytes = a_bytes + BN * kTmaChunk;
+    const int b_bytes = p.BN * 128;
+    const int stage_bytes = kBoxBytes + b_bytes;   // 1024-byte multiples: BN is a multiple of 16
+    uint8_t *epi = base + NST * stage_bytes;
+    uint8_t *raw = epi + kStoreWarps * 4096;       // a storing warp holds 32 rows of 128 bytes
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int set = blockIdx.z;
-    const int64_t m0 = (int64_t)blockIdx.x * kTcBM;
-    const int n0 = blockIdx.y * BN;
-    E *out = p.out + set * p.stride;
-    const uint32_t tcols = BN <= 32 ? 32u : (BN <= 64 ? 64u : (BN <= 128 ? 128u : 256u));
-    uint32_t crank = 0;
-    if (CL > 1) asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(crank));
-    const uint16_t cmask = (uint16_t)((1u << CL) - 1u);
-    if (warp == 0) {
-        tmem_alloc(smem_addr(&tmem_base_sh), tcols);
+    const uint32_t acols = p.BN <= 32 ? 32u : (p.BN <= 64 ? 64u : (p.BN <= 128 ? 128u : 256u));
+    if (warp == 3) {
+        tmem_alloc(smem_addr(&tmem_base_sh), 2 * acols);
         tmem_relinquish();
     }
-    if (tid == 32) {
+    if (tid == 0) {
         for (int i = 0; i < NST; ++i) {
-            mbar_init(smem_addr(&full[i]), 1);
-            mbar_init(smem_addr(&empty[i]), CL);
+            mbar_init(smem_addr(&full[i]), FILL ? 1 + kConvertWarps : 1);
+            mbar_init(smem_addr(&empty[i]), 1);
         }
-        mbar_init(smem_addr(&done), 1);
+        for (int i = 0; i < kRawBoxes; ++i) {
+            mbar_init(smem_addr(&rfull[i]), 1);
+            mbar_init(smem_addr(&rempty[i]), kConvertWarps);
+        }
+        for (int i = 0; i < 2; ++i) {
+            mbar_init(smem_addr(&afull[i]), 1);
+            mbar_init(smem_addr(&aempty[i]), kStoreWarps);
+        }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     tc_fence_before();
     __syncthreads();
-    if (CL > 1) cluster_sync_all();      // every member's barriers exist before any multicast
     tc_fence_after();
     const uint32_t tmem = tmem_base_sh;
-    const int nchunks = (p.K + KC - 1) / KC;
-    const uint32_t idesc = instr_desc(EB == 4 ? 2u : 1u, kTcBM, (uint32_t)BN);
-    const uint32_t stage_tx = (uint32_t)stage_bytes;
-    int failed = 0;
-    if (tid == 0) {
-        // producer
-        for (int c = 0; c < nchunks && !failed; ++c) {
-            const int s = c % NST;
-            if (c >= NST && !mbar_wait(smem_addr(&empty[s]), (uint32_t)(((c / NST) - 1) & 1))) {
-                failed = 1;
-                break;
+    const int nch = (p.K + KC - 1) / KC;
+    // a wait that gives up ends its role; the others give up on their own waits
+    auto failed = [&] { atomicExch(p.err, 1); };
+    auto stage_a = [&](int s) { return smem_addr(base + s * stage_bytes); };
+
+    if (tid == 0 || (RAW && tid == 64)) {
+        // loads: thread 0 fills the stages, A's boxes and B's; when A is
+        // rounded it fills the landing boxes and thread 64 the B of the stages
+        const bool do_raw = RAW && tid == 0;
+        int s = 0, n_issued = 0;
+        uint32_t ph = 0;
+        bool ok = true;
+        const int step = FILL ? 0 : p.w / EB, boxes = FILL ? 0 : 128 / p.w;
+        const int steps = do_raw ? nch * RPC : nch;
+        for (TileWalk t(p); t.more() && ok; t.next()) {
+            const int m0 = t.m * kTcBM, n0 = t.n * p.BN, set = t.set;
+            int u = 0, h = 0;
+            for (int c = 0; c < steps && ok; ++c) {
+                if (do_raw) {
+                    ok = mbar_wait(smem_addr(&rempty[s]), ph ^ 1);
+                    if (!ok) break;
+                    const uint32_t fb = smem_addr(&rfull[s]);
+                    mbar_expect_tx(fb, kBoxBytes);
+                    tma_load3(smem_addr(raw + s * kBoxBytes), &tmA, c * 32, m0, set, fb);
+                    if (++s == kRawBoxes) { s = 0; ph ^= 1; }
+                } else {
+                    ok = mbar_wait(smem_addr(&empty[s]), ph ^ 1);
+                    if (!ok) break;
+                    const uint32_t fb = smem_addr(&full[s]);
+                    mbar_expect_tx(fb, (uint32_t)(FILL ? b_bytes : stage_bytes));
+                    const uint32_t sa = stage_a(s);
+                    for (int b = 0; b < boxes; ++b) {
+                        tma_load4(sa + (uint32_t)(b * p.w * kTcBM), &tmA, h, m0, u, set, fb);
+                        h += step;
+                        if (h >= p.Kh) { h = 0; ++u; }
+                    }
+                    tma_load3(sa + kBoxBytes, &tmB, c * KC, n0, set, fb);
+                    if (++s == NST) { s = 0; ph ^= 1; }
+                }
+                ++n_issued;
             }
-            const uint32_t fb = smem_addr(&full[s]);
-            mbar_expect_tx(fb, stage_tx);
-            const uint32_t sa = smem_addr(base + s * stage_bytes), sb = sa + a_bytes;
-#pragma unroll
-            for (int cu = 0; cu < UNITS; ++cu) {
-                const int k = c * KC + cu * EPU;
-                const int ku = k / p.Kh, kh = k - ku * p.Kh;
-                tma_load4(sa + cu * (kTcBM * 16), &tmA, kh, (int)m0, ku, set, fb);
-                if (CL == 1)
-                    tma_load3(sb + cu * (BN * 16), &tmB, k, n0, set, fb);
-                else if (cu % CL == (int)crank)
-                    tma_load3_mc(sb + cu * (BN * 16), &tmB, k, n0, set, fb, cmask);
+        }
+        if (!ok) {
+            failed();
+            // the copies in flight land before the block may end
+            const int slots = do_raw ? kRawBoxes : NST;
+            for (int i = 0; i < slots && i < n_issued; ++i) {
+                if (--s < 0) { s = slots - 1; ph ^= 1; }
+                mbar_wait(smem_addr(do_raw ? &rfull[s] : &full[s]), ph);
             }
         }
     } else if (tid == 32) {
-        // MMA issuer
-        for (int c = 0; c < nchunks; ++c) {
-            const int s = c % NST;
-            if (!mbar_wait(smem_addr(&full[s]), (uint32_t)((c / NST) & 1))) {
-                failed = 1;
-                break;
-            }
-            tc_fence_after();
-            const uint32_t sa = smem_addr(base + s * stage_bytes), sb = sa + a_bytes;
+        // MMAs
+        const uint32_t idesc = instr_desc(EB == 4 ? 2u : 1u, kTcBM, (uint32_t)p.BN);
+        const int w = FILL ? 128 : p.w;
+        uint64_t ad[4], bd[4];                     // descriptors of the four K steps in stage 0
 #pragma unroll
-            for (int ks = 0; ks < UNITS / 2; ++ks) {
-                const uint64_t ad = smem_desc(sa + ks * 2 * (kTcBM * 16), kTcBM * 16, 128);
-                const uint64_t bd = smem_desc(sb + ks * 2 * (BN * 16), (uint32_t)(BN * 16), 128);
-                tc_mma<EB>(tmem, ad, bd, idesc, (c > 0 || ks > 0) ? 1u : 0u);
-            }
-            if (CL == 1) tc_commit(smem_addr(&empty[s]));
-            else tc_commit_mc(smem_addr(&empty[s]), cmask);
+        for (int ks = 0; ks < 4; ++ks) {
+            const int o = ks * 32;
+            const uint32_t at = w == 16 ? (uint32_t)(o * kTcBM) : (uint32_t)(o / w * w * kTcBM + o % w);
+            ad[ks] = tile_desc(stage_a(0) + at, w);
+            bd[ks] = tile_desc(stage_a(0) + kBoxBytes + o, 128);
         }
-        if (!failed) tc_commit(smem_addr(&done));
-    }
-    // everyone: the accumulator is complete once `done` fires
-    bool ok = __syncthreads_or(failed) == 0;
-    if (ok) ok = mbar_wait(smem_addr(&done), 0u);
-    ok = __syncthreads_and(ok) != 0;
-    tc_fence_after();
-    const float mx_in = __uint_as_float((unsigned)p.max_in[set]);
-    const int e_in = mx_in > 0.f ? ilogbf(mx_in) : 0;
-    const float sc = ldexpf(1.f, -e_in);
-    if (blockIdx.x == 0 && blockIdx.y == 0 && tid == 0) {
-        p.log2s[set] += e_in;
-        p.max_clear[set] = 0ull;
-    }
-    float mx = 0.f;
-    if (ok) {
-        constexpr int SW = 64, SP = SW + 4;
-        float *st = reinterpret_cast<float *>(base);
-        for (int c0 = 0; c0 < BN; c0 += SW) {
+        int s = 0;
+        uint32_t ph = 0, it = 0;
+        bool ok = true;
+        for (TileWalk t(p); t.more() && ok; t.next(), ++it) {
+            const uint32_t acc = tmem + (it & 1) * acols;
+            ok = mbar_wait(smem_addr(&aempty[it & 1]), ((it >> 1) & 1) ^ 1);
+            for (int c = 0; c < nch && ok; ++c) {
+                ok = mbar_wait(smem_addr(&full[s]), ph);
+                if (!ok) break;
+                tc_fence_after();
+                const uint64_t so = (uint64_t)((s * stage_bytes) >> 4);
 #pragma unroll
-            for (int q = 0; q < SW; q += 16) {
-                uint32_t r[16];
-                tmem_ld16(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)(c0 + q), r);
-#pragma unroll
-                for (int j = 0; j < 16; ++j) st[(warp * 32 + lane) * SP + q + j] = __uint_as_float(r[j]) * sc;
+                for (int ks = 0; ks < 4; ++ks)
+                    tc_mma<EB>(acc, ad[ks] + so, bd[ks] + so, idesc, (c > 0 || ks > 0) ? 1u : 0u);
+                tc_commit(smem_addr(&empty[s]));
+                if (++s == NST) { s = 0; ph ^= 1; }
             }
-            __syncthreads();
-            for (int i = tid; i < kTcBM * SW; i += kTcThreads) {
-                const int rr = i / SW, cc = i % SW;
-                const int64_t row = m0 + rr;
-                const int col = n0 + c0 + cc;
-                if (row < p.R && col < p.N) {
-                    const E v = round_elem<E>(st[rr * SP + cc]);
-                    out[row * p.N + col] = v;
-                    mx = fmaxf(mx, fabsf(elem_to_float<E>(v)));
+            if (ok) tc_commit(smem_addr(&afull[it & 1]));
+        }
+        if (!ok) failed();
+    } else if (warp >= 4 && warp < kConvert0) {
+        // results: tensor memory -> registers -> this warp's 32 x 128-byte
+        // buffer (16-byte units swizzled by the row) -> whole row segments
+        constexpr int CW = 128 / OB;               // columns per round
+        uint8_t *buf = epi + (warp - 4) * 4096;
+        const int rows0 = (warp & 3) * 32;         // the tensor-memory lanes of this warp
+        uint32_t it = 0;
+        bool ok = true;
+        int e_in = 0, scaled_set = -1;
+        float sc = 1.f;
+        for (TileWalk t(p); t.more(); t.next(), ++it) {
+            const int n = t.n, set = t.set;
+            const int64_t m0 = (int64_t)t.m * kTcBM + rows0;
+            float mx = 0.f;
+            if (!RAW) {
+                // the scale of this step: 2^-e_in, e_in the exponent of the input's largest |entry|
+                if (set != scaled_set) {
+                    const float mx_in = __uint_as_float((unsigned)p.max_in[set]);
+                    e_in = mx_in > 0.f ? ilogbf(mx_in) : 0;
+                    sc = ldexpf(1.f, -e_in);
+                    scaled_set = set;
+                }
+                if (n == 0 && t.m == 0 && tid == 128) {
+                    p.log2s[set] += e_in;
+                    p.max_clear[set] = 0ull;
                 }
             }
-            __syncthreads();
+            ok = mbar_wait(smem_addr(&afull[it & 1]), (it >> 1) & 1);
+            ok = __all_sync(0xffffffffu, ok);
+            if (!ok) break;
+            tc_fence_after();
+            const uint32_t acc = tmem + (it & 1) * acols + ((uint32_t)rows0 << 16);
+            uint8_t *out = static_cast<uint8_t *>(p.out) + ((int64_t)set * p.strideC) * OB;
+            for (int c0 = (warp - 4) / 4 * CW; c0 < p.BN; c0 += kStoreWarps / 4 * CW) {
+#pragma unroll
+                for (int h = 0; h < CW; h += 32) {
+                    if (h > 0 && c0 + h >= (int)acols) break;
+                    uint32_t v[32];
+                    tmem_ld32(acc + (uint32_t)(c0 + h), v);
+                    const bool whole = c0 + h + 32 <= p.BN;    // else 16 columns: BN is a multiple of 16
+                    if (OB == 4) {
+                        if (!RAW) {
+#pragma unroll
+                            for (int j = 0; j < 32; ++j) {
+                                v[j] = to_tf32(__uint_as_float(v[j]) * sc);
+                                if (j < 16 || whole) mx = fmaxf(mx, fabsf(__uint_as_float(v[j])));
+                            }
+                        }
+#pragma unroll
+                        for (int q = 0; q < 8; ++q)
+                            *reinterpret_cast<uint4 *>(buf + lane * 128 + ((q ^ (lane & 7)) * 16)) =
+                                make_uint4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
+                    } else {
+                        uint32_t x[16];
+#pragma unroll
+                        for (int j = 0; j < 16; ++j) {
+                            const __nv_bfloat162 b2 = __floats2bfloat162_rn(__uint_as_float(v[2 * j]) * sc,
+                                                                            __uint_as_float(v[2 * j + 1]) * sc);
+                            if (j < 8 || whole)
+                                mx = fmaxf(mx, fmaxf(fabsf(__low2float(b2)), fabsf(__high2float(b2))));
+                            x[j] = *reinterpret_cast<const uint32_t *>(&b2);
+                        }
+#pragma unroll
+                        for (int q = 0; q < 4; ++q)
+                            *reinterpret_cast<uint4 *>(buf + lane * 128 + (((h / 8 + q) ^ (lane & 7)) * 16)) =
+                                make_uint4(x[4 * q], x[4 * q + 1], x[4 * q + 2], x[4 * q + 3]);
+                    }
+                }
+                __syncwarp();
+                constexpr int EPO = 16 / OB;
+                const int unit = lane & 7;
+                const int col = n * p.BN + c0 + unit * EPO;
+                const int left = min(p.N, (n + 1) * p.BN) - col;
+                const int row1 = lane >> 3;                     // rows row1, row1 + 4, ...
+                uint8_t *dst = out + ((m0 + row1) * p.ldc + col) * OB;
+                const int64_t hop = 4 * p.ldc * OB;
+                const int rows = (int)min((int64_t)32, p.M - m0);
+                if (p.vec && left >= EPO) {
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) {
+                        const int rr = i * 4 + row1;
+                        const uint4 v = *reinterpret_cast<const uint4 *>(buf + rr * 128 + ((unit ^ (rr & 7)) * 16));
+                        if (rr < rows) *reinterpret_cast<uint4 *>(dst + i * hop) = v;
+                    }
+                } else {
+                    for (int i = 0; i < 8; ++i) {
+                        const int rr = i * 4 + row1;
+                        if (rr >= rows) break;
+                        const uint8_t *src = buf + rr * 128 + ((unit ^ (rr & 7)) * 16);
+                        for (int j = 0; j < EPO && j < left; ++j) {
+                            if (OB == 4) reinterpret_cast<uint32_t *>(dst + i * hop)[j] = reinterpret_cast<const uint32_t *>(src)[j];
+                            else reinterpret_cast<uint16_t *>(dst + i * hop)[j] = reinterpret_cast<const uint16_t *>(src)[j];
+                        }
+                    }
+                }
+                __syncwarp();
+            }
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(smem_addr(&aempty[it & 1]));
+            if (!RAW) {
+                for (int off = 16; off > 0; off >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, off));
+                if (lane == 0 && mx > 0.f) atomicMax(p.max_out + set, (unsigned long long)__float_as_uint(mx));
+            }
         }
-    } else if (tid == 0) {
-        atomicExch(p.err, 1);
+        if (!ok && lane == 0) failed();
+    } else if (SRC == kGather && warp >= kConvert0) {
+        // running tensor -> operand stage: a row per lane, four of the eight
+        // 16-byte units of its 128 bytes per thread
+        using E = typename std::conditional<EB == 4, uint32_t, uint16_t>::type;
+        constexpr int EPU = 16 / EB;
+        const int cw = warp - kConvert0, row = (cw & 3) * 32 + lane, u0 = (cw >> 2) * 4;
+        int s = 0;
+        uint32_t ph = 0;
+        bool ok = true;
+        // the values of one chunk of one tile; zeros past the rows and past K
+        auto load = [&](const TileWalk &t, int c, E (&v)[4][EPU]) {
+            const int64_t m = (int64_t)t.m * kTcBM + row;
+            const E *S = static_cast<const E *>(p.S) + t.set * p.strideC + m * p.Kh;
+            int k = c * KC + u0 * EPU;
+            int u = k / p.Kh, h = k - u * p.Kh;
+            const E *at = S + (int64_t)u * p.M * p.Kh;
+            const int64_t hop = p.M * p.Kh;
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+#pragma unroll
+                for (int j = 0; j < EPU; ++j) {
+                    v[q][j] = (m < p.M && k < p.K) ? __ldg(at + h) : (E)0;
+                    ++k;
+                    if (++h == p.Kh) { h = 0; at += hop; }
+                }
+        };
+        TileWalk t(p);
+        int c = 0;
+        __align__(16) E v[4][EPU], w[4][EPU];
+        if (t.more()) load(t, 0, v);
+        while (t.more()) {
+            // the next chunk's loads run while this one waits for its stage
+            TileWalk t1 = t;
+            int c1 = c + 1;
+            if (c1 == nch) { c1 = 0; t1.next(); }
+            if (t1.more()) load(t1, c1, w);
+            ok = __all_sync(0xffffffffu, mbar_wait(smem_addr(&empty[s]), ph ^ 1));
+            if (!ok) break;
+            uint8_t *op = base + s * stage_bytes + row * 128;
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+                *reinterpret_cast<uint4 *>(op + (((u0 + q) ^ (row & 7)) * 16)) = *reinterpret_cast<const uint4 *>(v[q]);
+            fence_proxy_async();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(smem_addr(&full[s]));
+            if (++s == NST) { s = 0; ph ^= 1; }
+            t = t1;
+            c = c1;
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+#pragma unroll
+                for (int j = 0; j < EPU; ++j) v[q][j] = w[q][j];
+        }
+        if (!ok && lane == 0) failed();
+    } else if (RAW && warp >= kConvert0) {
+        // rounding: landing box -> operand stage, both 128-byte rows with the
+        // copy engine's swizzle (16-byte unit c of row r at c ^ (r & 7))
+        const int cw = warp - kConvert0;
+        int s = 0, rs = 0;
+        uint32_t ph = 0, rph = 0;
+        bool ok = true;
+        for (TileWalk t(p); t.more() && ok; t.next()) {
+            for (int c = 0; c < nch && ok; ++c) {
+                ok = __all_sync(0xffffffffu, mbar_wait(smem_addr(&empty[s]), ph ^ 1));
+                if (!ok) break;
+                uint8_t *op = base + s * stage_bytes;
+#pragma unroll
+                for (int bx = 0; bx < RPC; ++bx) {
+                    ok = __all_sync(0xffffffffu, mbar_wait(smem_addr(&rfull[rs]), rph));
+                    if (!ok) break;
+                    const uint8_t *src = raw + rs * kBoxBytes;
+                    if (EB == 4) {
+                        // the same unit of the same row: the same offset
+                        for (int o = (cw * 32 + lane) * 16; o < kBoxBytes; o += kConvertWarps * 512) {
+                            const float4 f = *reinterpret_cast<const float4 *>(src + o);
+                            *reinterpret_cast<uint4 *>(op + o) =
+                                make_uint4(to_tf32(f.x), to_tf32(f.y), to_tf32(f.z), to_tf32(f.w));
+                        }
+                    } else {
+                        // eight values (two units of the box) to one unit; the rows of
+                        // a quarter warp differ by 5 mod 8, so that neither the reads
+                        // nor the writes meet in a bank
+                        const int k4 = lane & 3, r8 = (lane >> 3) ^ ((lane & 4) ? 5 : 0);
+                        for (int g = cw; g < kTcBM / 8; g += kConvertWarps) {
+                            const int r = g * 8 + r8;
+                            const float4 f = *reinterpret_cast<const float4 *>(src + r * 128 + (((2 * k4) ^ r8) * 16));
+                            const float4 h = *reinterpret_cast<const float4 *>(src + r * 128 + (((2 * k4 + 1) ^ r8) * 16));
+                            const __nv_bfloat162 a = __floats2bfloat162_rn(f.x, f.y), b = __floats2bfloat162_rn(f.z, f.w);
+                            const __nv_bfloat162 d = __floats2bfloat162_rn(h.x, h.y), e = __floats2bfloat162_rn(h.z, h.w);
+                            *reinterpret_cast<uint4 *>(op + r * 128 + (((bx * 4 + k4) ^ r8) * 16)) =
+                                make_uint4(*reinterpret_cast<const uint32_t *>(&a), *reinterpret_cast<const uint32_t *>(&b),
+                                           *reinterpret_cast<const uint32_t *>(&d), *reinterpret_cast<const uint32_t *>(&e));
+                        }
+                    }
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(smem_addr(&rempty[rs]));
+                    if (++rs == kRawBoxes) { rs = 0; rph ^= 1; }
+                }
+                if (!ok) break;
+                fence_proxy_async();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(smem_addr(&full[s]));
+                if (++s == NST) { s = 0; ph ^= 1; }
+            }
+        }
+        if (!ok && lane == 0) failed();
     }
-    for (int off = 16; off > 0; off >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, off));
-    if (lane == 0 && mx > 0.f) atomicMax(p.max_out + set, (unsigned long long)__float_as_uint(mx));
+    __syncwarp();
     tc_fence_before();
     __syncthreads();
-    if (warp == 0) tmem_dealloc(tmem, tcols);
-    if (CL > 1) cluster_sync_all();      // no member leaves while another may still signal it
+    if (warp == 3) tmem_dealloc(tmem, 2 * acols);
+}
+
+// B of pne_dense_gemm rounded to the operand type once, rows padded with zeros
+// to 16-byte units: W[b][n][ldw].  Each value is read again by every row tile,
+// so rounding it there would cost M / 128 times the work.
+template <int EB>
+__global__ void round_rows_kernel(const float *B, int64_t ldb, int64_t strideB, int N, int K, int ldw, void *W,
+                                  int64_t total)
+{
+    constexpr int EPU = 16 / EB;
+    const int units = ldw / EPU;
+    for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < total; q += (int64_t)gridDim.x * blockDim.x) {
+        const int u = (int)(q % units);
+        const int64_t r = q / units;
+        const float *row = B + r / N * strideB + r % N * ldb;
+        static_cast<uint4 *>(W)[q] = load_unit<EB>(row, u * EPU, K, true);
+    }
 }
 
 PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder()
@@ -967,110 +1081,93 @@ PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder()
     return fn;
 }
 
-template <typename E, int NST, int CL>
-cudaError_t launch_tma_n(const RingParams<E> &p, int batch, int BN, int n_sets, cudaStream_t s, bool &used)
+// tiles of BN <= 256 columns of equal width; narrower ones while the tiles
+// do not reach every SM (128 x 2048 x 256 TF32: 75 -> 18 us)
+void stream_tiles(StreamParams &p, int n_sm)
 {
-    used = false;
+    p.mt = (int)((p.M + kTcBM - 1) / kTcBM);
+    p.nt = (p.N + 255) / 256;
+    auto width = [&] { return ((p.N + p.nt - 1) / p.nt + 15) / 16 * 16; };
+    while ((int64_t)p.mt * p.nt * p.batch < n_sm && width() > 64) p.nt *= 2;
+    p.BN = width();
+    p.nt = (p.N + p.BN - 1) / p.BN;
+}
+
+template <int EB, int SRC>
+cudaError_t launch_stream(const CUtensorMap &ma, const CUtensorMap &mb, StreamParams p, int n_sm, cudaStream_t s)
+{
+    const int fixed = store_warps(SRC) * 4096 + (SRC == kRound ? kRawBoxes * kBoxBytes : 0) + 1024;
+    const int stage = kBoxBytes + p.BN * 128;
+    p.stages = std::min(kStreamStages, (226 * 1024 - fixed) / stage);   // 227 KB less the barriers
+    const size_t smem = (size_t)p.stages * stage + fixed;
+    cudaError_t e = grant_dynamic_smem((const void *)tc_stream_kernel<EB, SRC>, smem);
+    if (e != cudaSuccess) return e;
+    const int64_t tiles = (int64_t)p.mt * p.nt * p.batch;
+    tc_stream_kernel<EB, SRC><<<(unsigned)std::min<int64_t>(tiles, n_sm), stream_threads(SRC), smem, s>>>(ma, mb, p);
+    return cudaGetLastError();
+}
+
+// operand boxes of 128 bytes by `rows` rows over [batch][rows][ld]
+bool encode_rows(CUtensorMap *m, int eb, const void *ptr, int64_t ld, int64_t cols, int64_t rows, int64_t stride,
+                 int batch, int box_rows)
+{
     auto enc = tensor_map_encoder();
-    if (!enc) return cudaSuccess;
-    constexpr int EB = (int)sizeof(E);
-    const CUtensorMapDataType dt = EB == 4 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16;
-    CUtensorMap ma, mb;
-    // A: [set][Ku][R][Kh], innermost first
-    const cuuint64_t adim[4] = {(cuuint64_t)p.Kh, (cuuint64_t)p.R, (cuuint64_t)p.Ku, (cuuint64_t)n_sets};
-    const cuuint64_t astr[3] = {(cuuint64_t)p.Kh * EB, (cuuint64_t)p.R * p.Kh * EB, (cuuint64_t)p.stride * EB};
-    const cuuint32_t abox[4] = {(cuuint32_t)(16 / EB), (cuuint32_t)kTcBM, 1, 1};
-    const cuuint32_t one4[4] = {1, 1, 1, 1};
-    // B: [set][N][ldb]
-    const cuuint64_t bdim[3] = {(cuuint64_t)p.ldb, (cuuint64_t)p.N, (cuuint64_t)n_sets};
-    const cuuint64_t bstr[2] = {(cuuint64_t)p.ldb * EB, (cuuint64_t)p.b_stride * EB};
-    const cuuint32_t bbox[3] = {(cuuint32_t)(16 / EB), (cuuint32_t)BN, 1};
-    if (enc(&ma, dt, 4, (void *)p.S, adim, astr, abox, one4, CU_TENSOR_MAP_INTERLEAVE_NONE,
-            CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) !=
-            CUDA_SUCCESS ||
-        enc(&mb, dt, 3, (void *)p.B, bdim, bstr, bbox, one4, CU_TENSOR_MAP_INTERLEAVE_NONE,
-            CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) !=
-            CUDA_SUCCESS)
-        return cudaSuccess;         // not encodable: the copy-loop kernel runs instead
-    // the epilogue stages the accumulator through the same shared memory: 128 x 68 floats
-    const size_t smem = std::max<size_t>((size_t)NST * (kTcBM + BN) * kTmaChunk, (size_t)kTcBM * 68 * 4) + 1024;
-    cudaError_t e = grant_dynamic_smem((const void *)tc_tma_gemm_kernel<E, NST, CL>, smem);
-    if (e != cudaSuccess) return e;
-    const int64_t mt = (p.R + kTcBM - 1) / kTcBM;
-    const dim3 grid((unsigned)((mt + CL - 1) / CL * CL), (unsigned)((p.N + BN - 1) / BN), (unsigned)batch);
-    if (CL == 1) {
-        tc_tma_gemm_kernel<E, NST, CL><<<grid, kTcThreads, smem, s>>>(ma, mb, p, BN);
-    } else {
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = grid;
-        cfg.blockDim = dim3(kTcThreads, 1, 1);
-        cfg.dynamicSmemBytes = smem;
-        cfg.stream = s;
-        cudaLaunchAttribute attr[1];
-        attr[0].id = cudaLaunchAttributeClusterDimension;
-        attr[0].val.clusterDim.x = CL;
-        attr[0].val.clusterDim.y = 1;
-        attr[0].val.clusterDim.z = 1;
-        cfg.attrs = attr;
-        cfg.numAttrs = 1;
-        e = cudaLaunchKernelEx(&cfg, tc_tma_gemm_kernel<E, NST, CL>, ma, mb, p, BN);
-        if (e != cudaSuccess) return e;
-    }
-    used = true;
-    return cudaGetLastError();
+    if (!enc) return false;
+    const CUtensorMapDataType dt = eb == 4 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16;
+    const cuuint64_t dim[3] = {(cuuint64_t)cols, (cuuint64_t)rows, (cuuint64_t)batch};
+    const cuuint64_t str[2] = {(cuuint64_t)ld * eb, (cuuint64_t)(batch > 1 ? stride : ld * rows) * eb};
+    const cuuint32_t box[3] = {(cuuint32_t)(128 / eb), (cuuint32_t)box_rows, 1};
+    const cuuint32_t one[3] = {1, 1, 1};
+    return enc(m, dt, 3, const_cast<void *>(ptr), dim, str, box, one, CU_TENSOR_MAP_INTERLEAVE_NONE,
+               CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) ==
+           CUDA_SUCCESS;
 }
 
-// stages per CTA: as many as let two CTAs share an SM (<= 113 KB each, 2 x 256
-// tensor-memory columns), so one CTA's prologue and epilogue overlap the
-// other's main loop
-template <typename E, int NST>
-cudaError_t launch_ring_n(const RingParams<E> &p, int batch, int BN, cudaStream_t s)
-{
-    const size_t smem = (size_t)NST * (kATileBytes + BN * kChunk) + 1024;
-    cudaError_t e = grant_dynamic_smem((const void *)tc_ring_gemm_kernel<E, NST>, smem);
-    if (e != cudaSuccess) return e;
-    const dim3 grid((unsigned)((p.R + kTcBM - 1) / kTcBM), (unsigned)((p.N + BN - 1) / BN), (unsigned)batch);
-    tc_ring_gemm_kernel<E, NST><<<grid, kTcThreads, smem, s>>>(p, BN);
-    return cudaGetLastError();
-}
-
+// A site absorption on the persistent kernel.  The copy engine takes A where
+// every 16-byte unit of k is contiguous in the running tensor; the other sites
+// gather it.  The site matrix is padded to 16-byte rows (grid_plan).
 template <typename E>
-cudaError_t launch_ring(const RingParams<E> &p, int batch, cudaStream_t s)
+cudaError_t launch_grid_stream(const RingParams<E> &p, int batch, int n_sm, cudaStream_t s)
 {
-    const int BN = std::min(256, ((p.N + 15) / 16) * 16);
-    const int stage = kATileBytes + BN * kChunk;
-    const int nst = (int)std::max<int64_t>(2, std::min<int64_t>(4, (112 * 1024) / stage));
-    constexpr int EPU = 16 / (int)sizeof(E);
-    // TMA where every 16-byte unit of k is contiguous and every stride a multiple of 16 bytes
-    if (p.Kh % EPU == 0 && (p.ldb % EPU) == 0 && (p.stride % EPU) == 0 && (p.b_stride % EPU) == 0 &&
-        p.R < (int64_t)1 << 31) {
-        bool used = false;
-        // 64-byte stages: twice as many in flight in the same shared memory (two CTAs per SM)
-        const int tstage = (kTcBM + BN) * kTmaChunk;
-        const int tn = (int)std::max<int64_t>(2, std::min<int64_t>(8, (112 * 1024) / tstage));
-        // clusters of CL CTAs share the site matrix through multicast (PNE_TC_CLUSTER = 1, 2 or 4;
-        // default 2) when the rows fill at least two clusters
-        static const int cl_env = [] {
-            const char *v = std::getenv("PNE_TC_CLUSTER");
-            const int c = v ? std::atoi(v) : 2;
-            return (c == 1 || c == 2 || c == 4) ? c : 2;
-        }();
-        const int64_t mt = (p.R + kTcBM - 1) / kTcBM;
-        const int cl = mt >= 2 * cl_env ? cl_env : 1;
-        cudaError_t e;
-        if (cl == 4)
-            e = tn >= 8 ? launch_tma_n<E, 8, 4>(p, batch, BN, batch, s, used) : launch_tma_n<E, 4, 4>(p, batch, BN, batch, s, used);
-        else if (cl == 2)
-            e = tn >= 8 ? launch_tma_n<E, 8, 2>(p, batch, BN, batch, s, used) : launch_tma_n<E, 4, 2>(p, batch, BN, batch, s, used);
-        else
-            e = tn >= 8   ? launch_tma_n<E, 8, 1>(p, batch, BN, batch, s, used)
-                : tn >= 4 ? launch_tma_n<E, 4, 1>(p, batch, BN, batch, s, used)
-                          : launch_tma_n<E, 2, 1>(p, batch, BN, batch, s, used);
-        if (e != cudaSuccess || used) return e;
-    }
-    if (nst >= 4) return launch_ring_n<E, 4>(p, batch, BN, s);
-    if (nst == 3) return launch_ring_n<E, 3>(p, batch, BN, s);
-    return launch_ring_n<E, 2>(p, batch, BN, s);
+    auto enc = tensor_map_encoder();
+    if (!enc) return cudaErrorSymbolNotFound;
+    constexpr int EB = (int)sizeof(E);
+    StreamParams q{};
+    q.M = p.R;
+    q.N = p.N;
+    q.K = p.K;
+    q.batch = batch;
+    stream_tiles(q, n_sm);
+    q.Kh = p.Kh;
+    q.w = 128;
+    while (q.w > 16 && (p.Kh * EB) % q.w != 0) q.w /= 2;
+    q.out = p.out;
+    q.ldc = p.N;
+    q.strideC = p.stride;
+    q.vec = (p.N * EB) % 16 == 0 && (p.stride * EB) % 16 == 0 && (reinterpret_cast<uintptr_t>(p.out) & 15) == 0;
+    q.max_in = p.max_in;
+    q.max_out = p.max_out;
+    q.max_clear = p.max_clear;
+    q.log2s = p.log2s;
+    q.err = p.err;
+    q.S = p.S;
+    CUtensorMap ma{}, mb;
+    if (!encode_rows(&mb, EB, p.B, p.ldb, p.ldb, p.N, p.b_stride, batch, q.BN)) return cudaErrorInvalidValue;
+    if ((p.Kh * EB) % 16 != 0) return launch_stream<EB, kGather>(ma, mb, q, n_sm, s);
+    const CUtensorMapDataType dt = EB == 4 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16;
+    const CUtensorMapSwizzle sw = q.w == 128  ? CU_TENSOR_MAP_SWIZZLE_128B
+                                  : q.w == 64 ? CU_TENSOR_MAP_SWIZZLE_64B
+                                  : q.w == 32 ? CU_TENSOR_MAP_SWIZZLE_32B
+                                              : CU_TENSOR_MAP_SWIZZLE_NONE;
+    // A: [set][Ku][R][Kh], innermost first
+    const cuuint64_t adim[4] = {(cuuint64_t)p.Kh, (cuuint64_t)p.R, (cuuint64_t)p.Ku, (cuuint64_t)batch};
+    const cuuint64_t astr[3] = {(cuuint64_t)p.Kh * EB, (cuuint64_t)p.R * p.Kh * EB, (cuuint64_t)p.stride * EB};
+    const cuuint32_t abox[4] = {(cuuint32_t)(q.w / EB), (cuuint32_t)kTcBM, 1, 1};
+    const cuuint32_t one4[4] = {1, 1, 1, 1};
+    if (enc(&ma, dt, 4, (void *)p.S, adim, astr, abox, one4, CU_TENSOR_MAP_INTERLEAVE_NONE, sw,
+            CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+        return cudaErrorInvalidValue;
+    return launch_stream<EB, kBoxes>(ma, mb, q, n_sm, s);
 }
 
 size_t tc_smem_bytes(int BN)
@@ -1078,10 +1175,63 @@ size_t tc_smem_bytes(int BN)
     return (size_t)2 * (kATileBytes + BN * kChunk) + 1024;
 }
 
+// pne_dense_gemm on the persistent kernel, B rounded into `W` first; used =
+// false when A cannot be described to the copy engine
 template <int EB>
-cudaError_t launch_tc(const GemmParams<float> &p, int batch, cudaStream_t s)
+cudaError_t launch_dense_stream(const GemmParams<float> &p, int batch, int n_sm, void *W, int64_t ldw, cudaStream_t s,
+                                bool &used)
 {
+    used = false;
+    StreamParams q{};
+    q.M = p.M;
+    q.N = p.N;
+    q.K = p.K;
+    q.batch = batch;
+    stream_tiles(q, n_sm);
+    q.w = 128;
+    q.out = p.C;
+    q.ldc = p.ldc;
+    q.strideC = p.strideC;
+    q.vec = p.ldc % 4 == 0 && (batch == 1 || p.strideC % 4 == 0) && (reinterpret_cast<uintptr_t>(p.C) & 15) == 0;
+    q.err = p.err;
+    CUtensorMap ma, mb;
+    if (!encode_rows(&ma, 4, p.A, p.lda, p.K, p.M, p.strideA, batch, kTcBM) ||
+        !encode_rows(&mb, EB, W, ldw, ldw, p.N, ldw * p.N, batch, q.BN))
+        return cudaSuccess;
+    used = true;
+    const int64_t units = (int64_t)batch * p.N * (ldw / (16 / EB));
+    round_rows_kernel<EB><<<(unsigned)std::min<int64_t>((units + 255) / 256, (int64_t)n_sm * 16), 256, 0, s>>>(
+        p.B, p.ldb, p.strideB, p.N, p.K, (int)ldw, W, units);
+    const cudaError_t e = cudaGetLastError();
+    return e != cudaSuccess ? e : launch_stream<EB, kRound>(ma, mb, q, n_sm, s);
+}
+
+template <int EB>
+cudaError_t launch_tc(pne_ctx *ctx, const GemmParams<float> &p, int batch, cudaStream_t s)
+{
+    const bool aligned = (reinterpret_cast<uintptr_t>(p.A) & 15) == 0 && p.lda % 4 == 0 &&
+                         (batch == 1 || (p.strideA % 4 == 0 && p.strideA > 0));
     const int BN = std::min(256, ((p.N + 15) / 16) * 16);
+    // The copying kernel takes about K (128 + BN) loads per block, one by one;
+    // the persistent one costs a launch and a workspace more.  Whole calls
+    // cross between 64 x 64 x 64 (34.0 against 35.1 us TF32, 33.5 against 34.8
+    // BF16) and 512 x 128 x 128 (50.4 against 36.9, 46.4 against 35.2), BF16
+    // the later (16 x 640 x 64 x 100: 45.9 against 36.2 TF32, 34.6 against 35.8
+    // BF16); many blocks take it at any K.
+    const int64_t blocks = (int64_t)((p.M + kTcBM - 1) / kTcBM) * ((p.N + BN - 1) / BN) * batch;
+    const bool large = (int64_t)p.K * (kTcBM + BN) >= (EB == 4 ? 14000 : 20000) || blocks >= 2 * ctx->n_sm;
+    if (aligned && large) {
+        const int64_t ldw = ((int64_t)p.K * EB + 15) / 16 * 16 / EB;
+        DevBuf W;
+        if (dev_alloc(ctx, W, (size_t)batch * p.N * ldw * EB, s) == PNE_OK) {
+            bool used = false;
+            const cudaError_t e = launch_dense_stream<EB>(p, batch, ctx->n_sm, W.ptr, ldw, s, used);
+            dev_free(ctx, W, s);
+            if (e != cudaSuccess || used) return e;
+        } else {
+            (void)cudaGetLastError();     // no room for the workspace: the copying kernel needs none
+        }
+    }
     const size_t smem = tc_smem_bytes(BN);
     cudaError_t e = grant_dynamic_smem((const void *)tc_gemm_kernel<EB>, smem);
     if (e != cudaSuccess) return e;
@@ -1254,7 +1404,7 @@ pne_status grid_run(pne_ctx *ctx, const GridPlan &plan, const double *data, int6
                 rp.log2s = lg;
                 rp.err = (int *)dErr.ptr;
                 ProfScope ps(ctx, s, "grid_gemm_tc");
-                if ((ee = launch_ring<E>(rp, nb, s)) != cudaSuccess) return ee;
+                if ((ee = launch_grid_stream<E>(rp, nb, ctx->n_sm, s)) != cudaSuccess) return ee;
                 bound += 2.0 * u_in + (double)rp.K * std::ldexp(1.0, -24);
             }
             {
@@ -1346,7 +1496,7 @@ pne_status pne_dense_gemm(pne_ctx *ctx, pne_dtype dtype, int32_t batch, int32_t 
         } else {
             GemmParams<float> p{(const float *)A, lda, strideA, (const float *)B, ldb, strideB, (float *)C, ldc,
                                 strideC, M, N, K, nullptr, (int *)err.ptr};
-            e = dtype == PNE_TF32 ? launch_tc<4>(p, batch, s) : launch_tc<2>(p, batch, s);
+            e = dtype == PNE_TF32 ? launch_tc<4>(ctx, p, batch, s) : launch_tc<2>(ctx, p, batch, s);
         }
     }
     int herr = 0;
