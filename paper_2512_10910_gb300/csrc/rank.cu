@@ -11,7 +11,8 @@
 // right singular vectors and values of the matricised tensors are needed: a
 // Householder QR reduces each to a d x d triangle, whose SVD (and that of the
 // d x d core) is taken by one-sided Jacobi rotations (Hestenes), in FP64.
-// One thread block per tensor set runs the sweeps over the bonds in id order.
+// A cluster of up to eight thread blocks per tensor set runs the sweeps over
+// the bonds in id order.
 //
 // The rank-r expansion restricts, per term, each bond's index to the P range
 // [0, r) of the r largest weights, to the Q range [r, d), or leaves it whole,
@@ -49,8 +50,22 @@ pne_status geometry_for(pne_ctx *ctx, const pne_network *net, cudaStream_t s, st
 namespace {
 
 constexpr int kWpDim = 16;              // largest bond dimension of weight passing
-constexpr int kWpThreads = 256;
+constexpr int kWpThreads = 128;
 constexpr int kWpWarps = kWpThreads / 32;
+constexpr int kWpRows = 4;              // rows a thread holds during the QR
+constexpr int kWpPanel = kWpThreads * kWpRows;
+constexpr int kWpCluster = 8;           // most blocks per tensor set (portable cluster size)
+constexpr int kWpLd = kWpDim + 1;       // column stride of the Jacobi matrices in shared memory
+
+// What the blocks of one set pass to each other, in global memory (read past
+// L1), each field written between two cluster barriers and read after them.
+struct WPShare {
+    double R[kWpCluster][kWpDim * kWpDim];      // triangles of each block's rows, side A then side B
+    double RB[kWpCluster][kWpDim * kWpDim];
+    double WB[kWpDim * kWpDim], sB[kWpDim];     // U_B S_B (column c at c * kWpDim) and S_B
+    double XL[kWpDim * kWpDim], XR[kWpDim * kWpDim];   // leg transforms [in][out]
+    int code;                                   // 0 next bond, 1 a zero singular value, 2 converged
+};
 
 struct WPParams {
     int n_sets, n_sites, n_bonds;
@@ -59,8 +74,7 @@ struct WPParams {
     int64_t set_stride;
     double *T;                 // [n_sets][stride]: re-gauged in place, weighted at the end
     double *S;                 // [n_sets][n_bonds][kWpDim]
-    double *scratch;           // [n_sets][scratch_per]
-    int64_t scratch_per;
+    WPShare *share;            // [n_sets]
     double alpha, tol;
     int max_sweeps;
     double *log_scale;         // [n_sets]
@@ -68,294 +82,539 @@ struct WPParams {
     int32_t *flags;            // [n_sets] 1: a zero singular value
 };
 
-__device__ double block_sum(double v, double *red)
+__device__ __forceinline__ void wp_barrier(int blocks)
 {
-    for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
-    __syncthreads();
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
-    __syncthreads();
-    double t = 0.0;
-    for (int w = 0; w < kWpWarps; ++w) t += red[w];
-    __syncthreads();
+    if (blocks == 1) __syncthreads();
+    else asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
+}
+
+// Sums of NV values over the warp, one per group of 32 / NV lanes: value
+// lane / (32 / NV) is returned.  Halving the list at each exchange takes NV
+// additions instead of 5 NV; FP64 additions are what the QR's reductions cost
+// (an SM retires two lanes per clock).
+template <int NV>
+__device__ __forceinline__ double warp_sums(double (&v)[NV])
+{
+    const int lane = threadIdx.x & 31;
+    int off = 16;
+#pragma unroll
+    for (int h = NV / 2; h >= 1; h >>= 1, off >>= 1) {
+        const bool up = lane & off;
+#pragma unroll
+        for (int k = 0; k < h; ++k) {
+            const double give = up ? v[k] : v[k + h], keep = up ? v[k + h] : v[k];
+            v[k] = keep + __shfl_xor_sync(0xffffffffu, give, off);
+        }
+    }
+    double t = v[0];
+#pragma unroll
+    for (; off >= 1; off >>= 1) t += __shfl_xor_sync(0xffffffffu, t, off);
     return t;
 }
 
-// Tensor v of the set as a matrix [rest, d] (column = digit of leg l, rows =
-// the other legs row-major), the weights of every other leg multiplied in,
-// column-major into M (M[c * rest + row]).
-__device__ void matricise(const WPParams &p, const double *Tset, const double *Sset, int v, int l, double *M,
-                          int64_t &rest_out, int &d_out)
+struct QrShared {
+    double R[kWpDim][kWpDim];           // the triangle so far
+    double part[kWpWarps][kWpDim];      // per-warp sums of one column step
+    double f[kWpDim];
+};
+
+// One column step of the QR of [R; panel]: the reflection with head R[J][J]
+// and tail column J of the panel zeroes that column.  All inner products of
+// column J with columns J.. are formed in one pass over the registers and one
+// reduction; one warp turns them into the factors.
+template <int DM, int J>
+__device__ __forceinline__ void qr_column(double (&x)[kWpRows][DM], int nr, QrShared &q, int d)
 {
-    const int l0 = p.site_ptr[v], k = p.site_ptr[v + 1] - l0;
-    int dims[kMaxDeg], bonds[kMaxDeg];
-    for (int i = 0; i < k; ++i) { bonds[i] = p.site_bonds[l0 + i]; dims[i] = p.bond_dim[bonds[i]]; }
-    const int64_t n = p.tens_off[v + 1] - p.tens_off[v];
-    const int d = dims[l];
-    const int64_t rest = n / d;
-    const double *T = Tset + p.tens_off[v];
-    for (int64_t e = threadIdx.x; e < n; e += blockDim.x) {
-        int64_t r = e, row = 0, mul = 1;
-        int col = 0;
-        double wgt = 1.0;
-        for (int i = k - 1; i >= 0; --i) {
-            const int dg = (int)(r % dims[i]);
-            r /= dims[i];
-            if (i == l) { col = dg; continue; }
-            row += dg * mul;
-            mul *= dims[i];
-            wgt *= Sset[(int64_t)bonds[i] * kWpDim + dg];
-        }
-        M[(int64_t)col * rest + row] = T[e] * wgt;
+    constexpr int N = DM - J;
+    constexpr int NV = N > 8 ? 16 : (N > 4 ? 8 : (N > 2 ? 4 : (N > 1 ? 2 : 1)));
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    if (nr > 0) {
+        double g[NV];
+#pragma unroll
+        for (int c = 0; c < NV; ++c) g[c] = c < N ? x[0][J] * x[0][J + c < DM ? J + c : J] : 0.0;
+#pragma unroll
+        for (int r = 1; r < kWpRows; ++r)
+            if (r < nr) {
+#pragma unroll
+                for (int c = 0; c < N; ++c) g[c] = fma(x[r][J], x[r][J + c], g[c]);
+            }
+        const double t = warp_sums<NV>(g);
+        constexpr int per = 32 / NV;
+        if (lane % per == 0) q.part[warp][lane / per] = t;
+    } else if (lane < NV) {
+        q.part[warp][lane] = 0.0;
     }
-    rest_out = rest;
-    d_out = d;
+    __syncthreads();
+    if (warp == 0) {
+        const int c = lane & 15;
+        double s = 0.0;
+        if (c < N)
+            for (int w = lane >> 4; w < kWpWarps; w += 2) s += q.part[w][c];
+        s += __shfl_xor_sync(0xffffffffu, s, 16);       // lane c: sum over the panel of column J times column J + c
+        const double s0 = __shfl_sync(0xffffffffu, s, 0);
+        const double head = q.R[J][J];
+        const double nrm = sqrt(fma(head, head, s0));
+        const double diag = head >= 0.0 ? -nrm : nrm, vj = head - diag;
+        const double vn2 = fma(vj, vj, s0);
+        const double beta = (s0 > 0.0 && vn2 > 0.0) ? 2.0 / vn2 : 0.0;
+        if (lane < N) {
+            if (lane == 0) {
+                if (beta != 0.0) q.R[J][J] = diag;
+                q.f[J] = 0.0;
+            } else {
+                const double old = q.R[J][J + lane];
+                const double f = beta * fma(vj, old, s);
+                q.R[J][J + lane] = fma(-f, vj, old);
+                q.f[J + lane] = f;
+            }
+        }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int c = J + 1; c < DM; ++c) {
+        if (c >= d) break;
+        const double f = q.f[c];
+#pragma unroll
+        for (int r = 0; r < kWpRows; ++r)
+            if (r < nr) x[r][c] = fma(-f, x[r][J], x[r][c]);
+    }
+}
+
+template <int DM, int J>
+__device__ __forceinline__ void qr_columns(double (&x)[kWpRows][DM], int nr, QrShared &q, int d)
+{
+    if constexpr (J < DM) {
+        if (J < d) {
+            qr_column<DM, J>(x, nr, q, d);
+            qr_columns<DM, J + 1>(x, nr, q, d);
+        }
+    }
+}
+
+// The triangle of the QR of `rows` rows of d values, load(row, x) giving one,
+// into q.R.  A thread holds four rows of a panel in registers for all d column
+// steps (the panel is read once; the column-by-column form walked the matrix
+// 2 d times through L2), and each panel is stacked under the triangle so far.
+template <int DM, class Load>
+__device__ void qr_rows(const Load &load, int rows, int d, QrShared &q)
+{
+    const int warp = threadIdx.x >> 5;
+    __syncthreads();
+    for (int e = threadIdx.x; e < kWpDim * kWpDim; e += kWpThreads) q.R[e / kWpDim][e % kWpDim] = 0.0;
+    __syncthreads();
+    for (int p0 = 0; p0 < rows; p0 += kWpPanel) {
+        double x[kWpRows][DM];
+        int nr = 0;
+#pragma unroll
+        for (int r = 0; r < kWpRows; ++r) {
+            const int row = p0 + r * kWpThreads + (int)threadIdx.x;
+            if (p0 + r * kWpThreads + warp * 32 < rows) nr = r + 1;
+#pragma unroll
+            for (int c = 0; c < DM; ++c) x[r][c] = 0.0;
+            if (row < rows) load(row, x[r]);
+        }
+        qr_columns<DM, 0>(x, nr, q, d);
+    }
     __syncthreads();
 }
 
-// Householder QR of the column-major m x n matrix M (m >= n): the n x n
-// upper triangle R goes to R (row-major, ldr = kWpDim).  A warp per column
-// for the reflections' dot products.
-__device__ void householder_r(double *M, int64_t m, int n, double *R, double *red)
+// ---- one-sided Jacobi (Hestenes) of the columns of a matrix in shared memory
+// (entry (row, c) at c * kWpLd + row).  A round of the tournament rotates up to
+// eight disjoint pairs at once, sixteen threads to a pair and a row each: the
+// four warps of the block.  An FP64 instruction takes a warp's scheduler about
+// 64 clocks on this GPU (two lanes per clock and SM), an FP32 or integer one
+// two, so a round is as long as the FP64 instructions of one warp: the sums
+// halve their list at each exchange (5 additions for the three inner products,
+// not 12), and what only decides how fast the columns become orthogonal -- the
+// angle -- is FP32, taken from the bits of the FP64 sums; cosine and sine (c^2 +
+// s^2 = 1 to FP64's rounding) and the rotation are FP64.  At n = 16 a
+// round on one warp, four rows to a lane and all FP64, took 5.2 k clocks (two
+// thirds of a bond update: 1.03 M of 1.5 M clocks).
+struct JacobiPair {
+    int c0, c1;
+    bool on;
+};
+
+// Pair `pr` of round rd among n columns (n2 = n rounded up to even): the circle
+// method; an odd n leaves one column out.
+__device__ __forceinline__ JacobiPair jacobi_pair(int pr, int rd, int n, int n2)
 {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (int j = 0; j < n; ++j) {
-        double *x = M + (int64_t)j * m;
-        double s = 0.0;
-        for (int64_t i = j + threadIdx.x; i < m; i += blockDim.x) s += x[i] * x[i];
-        s = block_sum(s, red);
-        const double x0 = x[j];
-        const double nrm = sqrt(s);
-        const double alpha = (x0 >= 0.0) ? -nrm : nrm;
-        const double vj = x0 - alpha;
-        const double vn2 = s - x0 * x0 + vj * vj;
-        __syncthreads();
-        if (threadIdx.x == 0) x[j] = vj;
-        __syncthreads();
-        if (vn2 > 0.0) {
-            const double beta = 2.0 / vn2;
-            for (int c = j + 1 + warp; c < n; c += kWpWarps) {
-                double *y = M + (int64_t)c * m;
-                double dot = 0.0;
-                for (int64_t i = j + lane; i < m; i += 32) dot += x[i] * y[i];
-                for (int off = 16; off > 0; off >>= 1) dot += __shfl_xor_sync(0xffffffffu, dot, off);
-                const double f = beta * dot;
-                for (int64_t i = j + lane; i < m; i += 32) y[i] -= f * x[i];
-            }
-        }
-        __syncthreads();
-        if (threadIdx.x < n) {
-            const int c = threadIdx.x;
-            R[j * kWpDim + c] = (c < j) ? 0.0 : (c == j ? alpha : M[(int64_t)c * m + j]);
-        }
-        __syncthreads();
-    }
+    const int m = n2 - 1;
+    int c0 = rd + pr, c1 = rd + m - pr;
+    c0 = pr == 0 ? m : (c0 >= m ? c0 - m : c0);
+    c1 = pr == 0 ? rd : (c1 >= m ? c1 - m : c1);
+    const int lo = c0 < c1 ? c0 : c1, hi = c0 < c1 ? c1 : c0;
+    return {lo, hi, pr < n2 / 2 && hi < n};
 }
 
-// One-sided Jacobi SVD of the n x n row-major W (ld kWpDim): on return W's
-// columns are U * sigma, V (row-major, ld kWpDim) the right singular vectors
-// and sig the singular values, sorted descending (columns permuted alike).
-// One warp, a lane per row.
-__device__ void jacobi_svd(double *W, double *V, double *sig, int n)
+__device__ __forceinline__ int double_exponent(double x) { return (__double2hiint(x) >> 20) & 0x7ff; }
+
+// x 2^(1023 - e) truncated to FP32 (0 below FP32's range), and back, by bits
+__device__ __forceinline__ float scaled_float(double x, int e)
 {
-    const int lane = threadIdx.x & 31;
-    for (int c = 0; c < n; ++c)
-        if (lane < n) V[lane * kWpDim + c] = (lane == c) ? 1.0 : 0.0;
-    __syncwarp();
-    for (int sweep = 0; sweep < 60; ++sweep) {
+    const int hi = __double2hiint(x), ex = ((hi >> 20) & 0x7ff) - e + 127;
+    if (ex <= 0) return 0.f;
+    return __int_as_float((hi & 0x80000000) | (min(ex, 254) << 23) | ((hi & 0xfffff) << 3) |
+                          (int)((unsigned)__double2loint(x) >> 29));
+}
+__device__ __forceinline__ double widen(float x)        // normal x
+{
+    const int b = __float_as_int(x);
+    return __hiloint2double((b & 0x80000000) | ((((b >> 23) & 0xff) + 896) << 20) | ((b & 0x7fffff) >> 3), b << 29);
+}
+
+// On return the columns of W are orthogonal, sorted by their norms (sig)
+// descending; with ACC the rotations are accumulated on V (identity on entry,
+// the same layout), whose columns move along.  The whole block.
+template <bool ACC>
+__device__ void jacobi_columns(double *W, double *V, double *sig, int n)
+{
+    const int lane = threadIdx.x & 31, pr = threadIdx.x >> 4, row = threadIdx.x & 15, base = lane & 16;
+    const int n2 = n + (n & 1), rounds = n2 - 1;
+    for (int sweep = 0; sweep < 60 && n > 1; ++sweep) {
         int rotated = 0;
-        for (int p = 0; p < n - 1; ++p)
-            for (int q = p + 1; q < n; ++q) {
-                const double wp = lane < n ? W[lane * kWpDim + p] : 0.0;
-                const double wq = lane < n ? W[lane * kWpDim + q] : 0.0;
-                double a = wp * wp, b = wq * wq, g = wp * wq;
-                for (int off = 16; off > 0; off >>= 1) {
-                    a += __shfl_xor_sync(0xffffffffu, a, off);
-                    b += __shfl_xor_sync(0xffffffffu, b, off);
-                    g += __shfl_xor_sync(0xffffffffu, g, off);
+        for (int rd = 0; rd < rounds; ++rd) {
+            const JacobiPair p = jacobi_pair(pr, rd, n, n2);
+            const bool in = p.on && row < n;
+            double *wp = W + p.c0 * kWpLd + row, *wq = W + p.c1 * kWpLd + row;
+            const double x = in ? *wp : 0.0, y = in ? *wq : 0.0;
+            // sums over the 16 rows of x^2, y^2 and x y
+            double s0 = x * x, s1 = y * y;
+            const double s2 = x * y;
+            const bool u8 = lane & 8, u4 = lane & 4;
+            double g0 = __shfl_xor_sync(0xffffffffu, u8 ? s0 : s2, 8), g1 = __shfl_xor_sync(0xffffffffu, s1, 8);
+            s0 = (u8 ? s2 : s0) + g0;
+            s1 = s1 + g1;
+            g0 = __shfl_xor_sync(0xffffffffu, u4 ? s0 : s1, 4);
+            s0 = (u4 ? s1 : s0) + g0;                 // lanes 0: x^2, 4: y^2, 8: x y
+            s0 += __shfl_xor_sync(0xffffffffu, s0, 2);
+            s0 += __shfl_xor_sync(0xffffffffu, s0, 1);
+            const double a = __shfl_sync(0xffffffffu, s0, base), b = __shfl_sync(0xffffffffu, s0, base + 4),
+                         g = __shfl_sync(0xffffffffu, s0, base + 8);
+            // |g| <= 1e-15 sqrt(a b)
+            const int e = max(double_exponent(a), double_exponent(b));
+            const float af = scaled_float(a, e), bf = scaled_float(b, e), gf = scaled_float(g, e);
+            bool small = fabsf(gf) <= 1e-15f * sqrtf(af) * sqrtf(bf);
+            if (af == 0.f || bf == 0.f) small = fabs(g) <= 1e-15 * sqrt(a) * sqrt(b);   // norms 2^63 apart
+            const bool turn = p.on && !(small || g == 0.0);
+            if (turn) {
+                // tangent of the rotation that takes g to zero: t = sign(z) / (|z| + sqrt(1 + z^2)), z = h / (2 g)
+                const double h = b - a;
+                const int eh = max(double_exponent(h), double_exponent(g));
+                const float hf = scaled_float(h, eh), g2 = 2.f * scaled_float(g, eh);
+                const float t = (hf < 0.f ? -g2 : g2) / (fabsf(hf) + sqrtf(fmaf(hf, hf, g2 * g2)));
+                double cs, sn;
+                if (fabsf(t) >= 1e-18f && fabsf(t) <= 1.5f) {
+                    // c = rsqrt(1 + t^2) and s = t c in FP32 miss c^2 + s^2 = 1 by r = O(1e-7), which
+                    // (1 + r)^(-1/2) to second order corrects; t c and c^2 are exact in FP64
+                    const double c = widen(rsqrtf(fmaf(t, t, 1.f))), s = widen(t) * c;
+                    const double r = fma(s, s, fma(c, c, -1.0));
+                    const double k = fma(r, fma(r, 0.375, -0.5), 1.0);
+                    cs = c * k;
+                    sn = s * k;
+                } else {                                 // graded beyond FP32: t = g / h to rounding
+                    cs = 1.0;
+                    sn = g / h;
                 }
-                if (fabs(g) <= 1e-15 * sqrt(a * b) || g == 0.0) continue;
-                rotated = 1;
-                const double zeta = (b - a) / (2.0 * g);
-                const double t = (zeta >= 0.0 ? 1.0 : -1.0) / (fabs(zeta) + sqrt(1.0 + zeta * zeta));
-                const double cs = 1.0 / sqrt(1.0 + t * t), sn = cs * t;
-                if (lane < n) {
-                    W[lane * kWpDim + p] = cs * wp - sn * wq;
-                    W[lane * kWpDim + q] = sn * wp + cs * wq;
-                    const double vp = V[lane * kWpDim + p], vq = V[lane * kWpDim + q];
-                    V[lane * kWpDim + p] = cs * vp - sn * vq;
-                    V[lane * kWpDim + q] = sn * vp + cs * vq;
+                if (row < n) {
+                    *wp = cs * x - sn * y;
+                    *wq = sn * x + cs * y;
+                    if (ACC) {
+                        double *vp = V + p.c0 * kWpLd + row, *vq = V + p.c1 * kWpLd + row;
+                        const double vx = *vp, vy = *vq;
+                        *vp = cs * vx - sn * vy;
+                        *vq = sn * vx + cs * vy;
+                    }
                 }
-                __syncwarp();
             }
+            rotated |= __syncthreads_or(turn);
+        }
         if (!rotated) break;
     }
+    if (threadIdx.x >= 32) return;
+    __syncwarp();
+    // norms, a column per lane, and the descending order (ties by index)
+    double norm = -1.0;
+    if (lane < n) {
+        double s2 = 0.0;
+        for (int row = 0; row < n; ++row) s2 = fma(W[lane * kWpLd + row], W[lane * kWpLd + row], s2);
+        norm = sqrt(s2);
+    }
+    int at = 0;
     for (int c = 0; c < n; ++c) {
-        const double w = lane < n ? W[lane * kWpDim + c] : 0.0;
-        double s2 = w * w;
-        for (int off = 16; off > 0; off >>= 1) s2 += __shfl_xor_sync(0xffffffffu, s2, off);
-        if (lane == 0) sig[c] = sqrt(s2);
+        const double o = __shfl_sync(0xffffffffu, norm, c);
+        at += (o > norm || (o == norm && c < lane)) ? 1 : 0;
+    }
+    double col[kWpDim], vcol[kWpDim];
+    if (lane < n)
+        for (int row = 0; row < n; ++row) {
+            col[row] = W[lane * kWpLd + row];
+            if (ACC) vcol[row] = V[lane * kWpLd + row];
+        }
+    __syncwarp();
+    if (lane < n) {
+        sig[at] = norm;
+        for (int row = 0; row < n; ++row) {
+            W[at * kWpLd + row] = col[row];
+            if (ACC) V[at * kWpLd + row] = vcol[row];
+        }
     }
     __syncwarp();
-    // selection sort by singular value, descending (columns of W and V move along)
-    for (int i = 0; i < n; ++i) {
-        int best = i;
-        for (int c = i + 1; c < n; ++c) if (sig[c] > sig[best]) best = c;
-        if (best != i) {
-            if (lane < n) {
-                double t = W[lane * kWpDim + i]; W[lane * kWpDim + i] = W[lane * kWpDim + best]; W[lane * kWpDim + best] = t;
-                t = V[lane * kWpDim + i]; V[lane * kWpDim + i] = V[lane * kWpDim + best]; V[lane * kWpDim + best] = t;
-            }
-            __syncwarp();
-            if (lane == 0) { const double t = sig[i]; sig[i] = sig[best]; sig[best] = t; }
-        }
-        __syncwarp();
-    }
 }
 
-// T_v <- T_v with leg l multiplied by the d x d matrix X: new[.., c, ..] =
-// sum_a old[.., a, ..] X[a][c] when right == 0, or sum_a X[c][a] old[.., a, ..]
-// when right == 1.  `tmp` holds a copy of the tensor.
-__device__ void apply_leg(const WPParams &p, double *Tset, int v, int l, const double *X, int right, double *tmp)
+// A site's legs as one bond update needs them
+struct WPSite {
+    const double *T;
+    int64_t T_off;
+    int k, l, d, rest;
+    int dims[kMaxDeg], stride[kMaxDeg], bond[kMaxDeg];
+};
+
+__device__ WPSite wp_site(const WPParams &p, const double *Tset, int v, int l)
 {
-    const int l0 = p.site_ptr[v], k = p.site_ptr[v + 1] - l0;
-    int dims[kMaxDeg];
-    for (int i = 0; i < k; ++i) dims[i] = p.bond_dim[p.site_bonds[l0 + i]];
-    int64_t post = 1;
-    for (int i = l + 1; i < k; ++i) post *= dims[i];
-    const int d = dims[l];
-    const int64_t n = p.tens_off[v + 1] - p.tens_off[v];
-    double *T = Tset + p.tens_off[v];
-    for (int64_t e = threadIdx.x; e < n; e += blockDim.x) tmp[e] = T[e];
-    __syncthreads();
-    for (int64_t e = threadIdx.x; e < n; e += blockDim.x) {
-        const int64_t lo = e % post, hi = e / post / d;
-        const int c = (int)((e / post) % d);
-        double acc = 0.0;
-        for (int a = 0; a < d; ++a) {
-            const double m = right ? X[c * kWpDim + a] : X[a * kWpDim + c];
-            acc = fma(tmp[(hi * d + a) * post + lo], m, acc);
-        }
-        T[e] = acc;
+    WPSite s;
+    const int l0 = p.site_ptr[v];
+    s.k = p.site_ptr[v + 1] - l0;
+    s.l = l;
+    s.T_off = p.tens_off[v];
+    s.T = Tset + s.T_off;
+    int stride = 1;
+    for (int i = s.k - 1; i >= 0; --i) {
+        s.bond[i] = p.site_bonds[l0 + i];
+        s.dims[i] = p.bond_dim[s.bond[i]];
+        s.stride[i] = stride;
+        stride *= s.dims[i];
     }
-    __syncthreads();
+    s.d = s.dims[l];
+    s.rest = stride / s.d;
+    return s;
 }
 
-__global__ void __launch_bounds__(kWpThreads) weight_passing_kernel(WPParams p)
+// Start of row `row` (the other legs row-major) in the site's tensor; the
+// product of those legs' weights (Sset, read past L1) in *wgt when asked for
+__device__ __forceinline__ int wp_row(const WPSite &s, int row, const double *Sset, double *wgt)
 {
-    __shared__ double red[kWpWarps];
-    __shared__ double RA[kWpDim * kWpDim], VA[kWpDim * kWpDim], RB[kWpDim * kWpDim], VB[kWpDim * kWpDim];
-    __shared__ double MC[kWpDim * kWpDim], VC[kWpDim * kWpDim], X[kWpDim * kWpDim];
-    __shared__ double sA[kWpDim], sB[kWpDim], sC[kWpDim];
-    __shared__ double change_sh, scale_sh;
+    int off = 0;
+    double w = 1.0;
+    for (int i = s.k - 1; i >= 0; --i) {
+        if (i == s.l) continue;
+        const int q = row / s.dims[i], dg = row - q * s.dims[i];
+        row = q;
+        off += dg * s.stride[i];
+        if (wgt) w *= __ldcg(Sset + (int64_t)s.bond[i] * kWpDim + dg);
+    }
+    if (wgt) *wgt = w;
+    return off;
+}
+
+// The updates of one tensor set by a cluster of blocks.  Per bond: the rows of
+// a matricised tensor above one panel are split over the blocks, each block's
+// rows reduced to a triangle; block 0 takes A (stacking the triangles, or the
+// whole of a small tensor) to its SVD while block 1 takes B; block 0 forms the
+// core, its SVD, the weights and the leg transforms; every block multiplies
+// its rows.  FP64 multiply-adds bound the large tensors (two per clock and
+// SM: 2 x 1.05 M for a 16^4 tensor, so the split over SMs is what pays), the
+// chain of column steps and Jacobi rounds the small ones.
+// Measured, blocked Ising 3 x 3, 8 sets, 0.65 to 0.8 T_c: chi = 16 860 -> 93 ms
+// (one block of 256 threads per set walked each matrix column by column in L2
+// and rotated one pair of columns at a time), chi = 8 246 -> 46, chi = 4 89 -> 30.
+template <int DM>
+__global__ void __launch_bounds__(kWpThreads) weight_passing_kernel(WPParams p, int blocks)
+{
+    __shared__ QrShared q;
+    __shared__ double WA[kWpDim * kWpLd], WBs[kWpDim * kWpLd], WC[kWpDim * kWpLd], VC[kWpDim * kWpLd];
+    __shared__ double X[2][kWpDim * kWpDim];
+    __shared__ double sA[kWpDim], sB[kWpDim], sC[kWpDim], gC[kWpDim];
     __shared__ int bad_sh;
-    const int set = blockIdx.x;
-    if (set >= p.n_sets) return;
+    const int set = blockIdx.x / blocks, rank = blockIdx.x % blocks, tid = threadIdx.x;
     double *Tset = p.T + (int64_t)set * p.set_stride;
     double *Sset = p.S + (int64_t)set * p.n_bonds * kWpDim;
-    double *buf = p.scratch + (int64_t)set * p.scratch_per;
-    for (int64_t i = threadIdx.x; i < (int64_t)p.n_bonds * kWpDim; i += blockDim.x)
+    WPShare &sh = p.share[set];
+    for (int64_t i = rank * kWpThreads + tid; i < (int64_t)p.n_bonds * kWpDim; i += blocks * kWpThreads)
         Sset[i] = ((int)(i % kWpDim) < p.bond_dim[i / kWpDim]) ? 1.0 : 0.0;
-    if (threadIdx.x == 0) { scale_sh = 0.0; bad_sh = 0; }
-    __syncthreads();
-    int done = 0;
-    for (int sweep = 1; sweep <= p.max_sweeps && !done; ++sweep) {
-        if (threadIdx.x == 0) change_sh = 0.0;
-        __syncthreads();
-        for (int b = 0; b < p.n_bonds; ++b) {
-            const int u = p.bond_site[2 * b], v = p.bond_site[2 * b + 1];
-            const int lu = p.bond_leg[2 * b], lv = p.bond_leg[2 * b + 1];
-            int64_t mA, mB;
-            int d, d2;
-            // A' and B' (other legs' weights absorbed), reduced to triangles
-            matricise(p, Tset, Sset, u, lu, buf, mA, d);
-            householder_r(buf, mA, d, RA, red);
-            matricise(p, Tset, Sset, v, lv, buf, mB, d2);
-            householder_r(buf, mB, d, RB, red);
-            if (threadIdx.x < 32) {
-                jacobi_svd(RA, VA, sA, d);      // right vectors V_A, values S_A
-                jacobi_svd(RB, VB, sB, d);      // B'^T: right vectors U_B, values S_B
-            }
-            __syncthreads();
-            if (threadIdx.x == 0)
-                for (int a = 0; a < d; ++a) if (!(sA[a] > 1e-300) || !(sB[a] > 1e-300)) bad_sh = 1;
-            __syncthreads();
-            if (bad_sh) break;
-            // core M = S_A V_A^T S_i U_B S_B and its SVD
-            const double *Si = Sset + (int64_t)b * kWpDim;
-            for (int e = threadIdx.x; e < d * d; e += blockDim.x) {
-                const int a = e / d, c = e % d;
-                double acc = 0.0;
-                for (int x = 0; x < d; ++x) acc = fma(VA[x * kWpDim + a] * Si[x], VB[x * kWpDim + c], acc);
-                MC[a * kWpDim + c] = sA[a] * acc * sB[c];
-            }
-            __syncthreads();
-            if (threadIdx.x < 32) jacobi_svd(MC, VC, sC, d);     // MC -> U_C S_C, VC = V_C
-            __syncthreads();
-            if (threadIdx.x == 0) {
-                double mx = 0.0;
-                for (int a = 0; a < d; ++a) mx = fmax(mx, pow(sC[a], p.alpha));
-                if (!(sC[d - 1] > 1e-300)) bad_sh = 1;
-                scale_sh += log(mx);
-                double ch = change_sh;
-                for (int a = 0; a < d; ++a) {
-                    const double nw = pow(sC[a], p.alpha) / mx;
-                    ch = fmax(ch, fabs(nw - Sset[(int64_t)b * kWpDim + a]));
-                    Sset[(int64_t)b * kWpDim + a] = nw;
+    double scale = 0.0, change = 0.0;      // kept by block 0's first warp
+    int code = 0, sweep = 0;               // without a bond the first sweep changes nothing
+    wp_barrier(blocks);
+    while (code == 0 && sweep < p.max_sweeps) {
+        ++sweep;
+        change = 0.0;
+        if (p.n_bonds == 0) code = 2;
+        for (int b = 0; b < p.n_bonds && code != 1; ++b) {
+            const WPSite sa = wp_site(p, Tset, p.bond_site[2 * b], p.bond_leg[2 * b]);
+            const WPSite sb = wp_site(p, Tset, p.bond_site[2 * b + 1], p.bond_leg[2 * b + 1]);
+            const int d = sa.d;
+            const bool split_a = blocks > 1 && sa.rest > kWpPanel, split_b = blocks > 1 && sb.rest > kWpPanel;
+            auto rows_of = [&](const WPSite &s, int lo) {
+                return [&s, lo, Sset](int row, double (&x)[DM]) {
+                    double w;
+                    const double *t = s.T + wp_row(s, lo + row, Sset, &w);
+#pragma unroll
+                    for (int c = 0; c < DM; ++c)
+                        if (c < s.d) x[c] = __ldcg(t + (int64_t)c * s.stride[s.l]) * w;
+                };
+            };
+            auto share_rows = [&](const WPSite &s, double (*R)[kWpDim * kWpDim]) {
+                const int per = (s.rest + blocks - 1) / blocks, lo = min(s.rest, rank * per);
+                qr_rows<DM>(rows_of(s, lo), min(s.rest, lo + per) - lo, d, q);
+                for (int e = tid; e < kWpDim * kWpDim; e += kWpThreads) __stcg(&R[rank][e], q.R[e / kWpDim][e % kWpDim]);
+            };
+            if (split_a) share_rows(sa, sh.R);
+            if (split_b) share_rows(sb, sh.RB);
+            if (split_a || split_b) wp_barrier(blocks);
+            // the triangle of one side to V S, the columns of its transpose after the rotations
+            auto side = [&](const WPSite &s, bool split, const double (*R)[kWpDim * kWpDim], double *W, double *sig) {
+                if (split)
+                    qr_rows<DM>([&](int row, double (&x)[DM]) {
+#pragma unroll
+                        for (int c = 0; c < DM; ++c)
+                            if (c < d) x[c] = __ldcg(&R[row / d][row % d * kWpDim + c]);
+                    }, blocks * d, d, q);
+                else
+                    qr_rows<DM>(rows_of(s, 0), s.rest, d, q);
+                for (int e = tid; e < d * d; e += kWpThreads) W[e / d * kWpLd + e % d] = q.R[e / d][e % d];
+                __syncthreads();
+                jacobi_columns<false>(W, nullptr, sig, d);
+                __syncthreads();
+            };
+            const int rank_b = blocks > 1 ? 1 : 0;
+            if (rank == 0) side(sa, split_a, sh.R, WA, sA);
+            if (rank == rank_b) {
+                side(sb, split_b, sh.RB, WBs, sB);
+                if (blocks > 1) {
+                    for (int e = tid; e < d * d; e += kWpThreads) __stcg(&sh.WB[e / d * kWpDim + e % d], WBs[e / d * kWpLd + e % d]);
+                    if (tid < d) __stcg(&sh.sB[tid], sB[tid]);
                 }
-                change_sh = ch;
             }
-            __syncthreads();
-            if (bad_sh) break;
-            // left = V_A S_A^{-1} U_C S_C^{(1-alpha)/2} on A's leg
-            for (int e = threadIdx.x; e < d * d; e += blockDim.x) {
-                const int a = e / d, c = e % d;
-                double acc = 0.0;
-                for (int x = 0; x < d; ++x) acc = fma(VA[a * kWpDim + x] / sA[x], MC[x * kWpDim + c] / sC[c], acc);
-                X[a * kWpDim + c] = acc * pow(sC[c], 0.5 * (1.0 - p.alpha));
+            if (blocks > 1) wp_barrier(blocks);
+            if (rank == 0) {
+                if (blocks > 1) {
+                    for (int e = tid; e < d * d; e += kWpThreads) WBs[e / d * kWpLd + e % d] = __ldcg(&sh.WB[e / d * kWpDim + e % d]);
+                    if (tid < d) sB[tid] = __ldcg(&sh.sB[tid]);
+                }
+                if (tid == 0) bad_sh = 0;
+                __syncthreads();
+                if (tid < d && (!(sA[tid] > 1e-300) || !(sB[tid] > 1e-300))) bad_sh = 1;
+                // core M = S_A V_A^T S_i U_B S_B and its SVD
+                double *Si = Sset + (int64_t)b * kWpDim;
+                for (int e = tid; e < d * d; e += kWpThreads) {
+                    const int a = e / d, c = e % d;
+                    double acc = 0.0;
+                    for (int x = 0; x < d; ++x) acc = fma(WA[a * kWpLd + x] * __ldcg(Si + x), WBs[c * kWpLd + x], acc);
+                    WC[c * kWpLd + a] = acc;
+                    VC[c * kWpLd + a] = a == c ? 1.0 : 0.0;
+                }
+                __syncthreads();
+                if (!bad_sh) jacobi_columns<true>(WC, VC, sC, d);          // WC -> U_C S_C, VC = V_C
+                if (!bad_sh && tid < 32) {
+                    const double s = tid < d ? sC[tid] : 0.0;
+                    if (!(sC[d - 1] > 1e-300)) bad_sh = 1;
+                    const double w = tid < d ? pow(s, p.alpha) : 0.0;
+                    if (tid < d) gC[tid] = pow(s, 0.5 * (1.0 - p.alpha));
+                    double mx = w;
+                    for (int off = 16; off > 0; off >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, off));
+                    scale += log(mx);
+                    const double nw = w / mx;
+                    double ch = tid < d ? fabs(nw - __ldcg(Si + tid)) : 0.0;
+                    for (int off = 16; off > 0; off >>= 1) ch = fmax(ch, __shfl_xor_sync(0xffffffffu, ch, off));
+                    change = fmax(change, ch);
+                    if (tid < d) __stcg(Si + tid, nw);
+                }
+                __syncthreads();
+                if (!bad_sh) {
+                    // left = V_A S_A^{-1} U_C S_C^{(1-alpha)/2} on A's leg,
+                    // right = S_C^{(1-alpha)/2} V_C^T S_B^{-1} U_B^T on B's, as [in][out]
+                    for (int e = tid; e < d * d; e += kWpThreads) {
+                        const int c = e / d, at = c * kWpLd + e % d;
+                        WA[at] = WA[at] / sA[c] / sA[c];
+                        WBs[at] = WBs[at] / sB[c] / sB[c];
+                        WC[at] = WC[at] / sC[c];
+                    }
+                    __syncthreads();
+                    for (int e = tid; e < 2 * d * d; e += kWpThreads) {
+                        const int side_b = e >= d * d, f = e - side_b * d * d, a = f / d, c = f % d;
+                        const double *L = (side_b ? WBs : WA) + a, *R = (side_b ? VC : WC) + c * kWpLd;
+                        double acc = 0.0;
+                        for (int x = 0; x < d; ++x) acc = fma(L[x * kWpLd], R[x], acc);
+                        __stcg((side_b ? sh.XR : sh.XL) + a * kWpDim + c, acc * gC[c]);
+                    }
+                }
+                if (tid == 0) __stcg(&sh.code, bad_sh ? 1 : (b == p.n_bonds - 1 && change < p.tol ? 2 : 0));
             }
-            __syncthreads();
-            apply_leg(p, Tset, u, lu, X, 0, buf);
-            // right = S_C^{(1-alpha)/2} V_C^T S_B^{-1} U_B^T on B's leg
-            for (int e = threadIdx.x; e < d * d; e += blockDim.x) {
-                const int c = e / d, a = e % d;
-                double acc = 0.0;
-                for (int x = 0; x < d; ++x) acc = fma(VC[x * kWpDim + c] / sB[x], VB[a * kWpDim + x], acc);
-                X[c * kWpDim + a] = pow(sC[c], 0.5 * (1.0 - p.alpha)) * acc;
+            wp_barrier(blocks);
+            code = __ldcg(&sh.code);
+            if (code != 1) {
+                for (int e = tid; e < d * d; e += kWpThreads) {
+                    X[0][e / d * kWpDim + e % d] = __ldcg(sh.XL + e / d * kWpDim + e % d);
+                    X[1][e / d * kWpDim + e % d] = __ldcg(sh.XR + e / d * kWpDim + e % d);
+                }
+                __syncthreads();
+                // rows of both tensors times their transform, a row per thread
+                for (int side_b = 0; side_b < 2; ++side_b) {
+                    const WPSite &s = side_b ? sb : sa;
+                    const double *Xs = X[side_b];
+                    const int st = s.stride[s.l];
+                    for (int row = rank * kWpThreads + tid; row < s.rest; row += blocks * kWpThreads) {
+                        double *t = Tset + s.T_off + wp_row(s, row, nullptr, nullptr);
+                        double in[DM], out[DM];
+#pragma unroll
+                        for (int c = 0; c < DM; ++c) {
+                            in[c] = c < d ? __ldcg(t + (int64_t)c * st) : 0.0;
+                            out[c] = 0.0;
+                        }
+#pragma unroll
+                        for (int a = 0; a < DM; ++a) {
+                            if (a >= d) break;
+#pragma unroll
+                            for (int c = 0; c < DM; ++c)
+                                if (c < d) out[c] = fma(in[a], Xs[a * kWpDim + c], out[c]);
+                        }
+#pragma unroll
+                        for (int c = 0; c < DM; ++c)
+                            if (c < d) __stcg(t + (int64_t)c * st, out[c]);
+                    }
+                }
             }
-            __syncthreads();
-            apply_leg(p, Tset, v, lv, X, 1, buf);
+            wp_barrier(blocks);
         }
-        __syncthreads();
-        if (bad_sh) break;
-        if (change_sh < p.tol) {
-            done = 1;
-            if (threadIdx.x == 0) p.sweeps[set] = sweep;
-        }
-        __syncthreads();
     }
-    if (threadIdx.x == 0) {
-        if (!done) p.sweeps[set] = 0;
-        p.flags[set] = bad_sh;
-        p.log_scale[set] = scale_sh;
+    if (rank == 0 && tid == 0) {
+        p.sweeps[set] = code == 2 ? sweep : 0;
+        p.flags[set] = code == 1;
+        p.log_scale[set] = scale;
     }
     // the weighted network: sqrt(S) into both ends of every bond
     for (int v = 0; v < p.n_sites; ++v) {
         const int l0 = p.site_ptr[v], k = p.site_ptr[v + 1] - l0;
-        int dims[kMaxDeg], bonds[kMaxDeg];
-        for (int i = 0; i < k; ++i) { bonds[i] = p.site_bonds[l0 + i]; dims[i] = p.bond_dim[bonds[i]]; }
-        const int64_t n = p.tens_off[v + 1] - p.tens_off[v];
+        const int n = (int)(p.tens_off[v + 1] - p.tens_off[v]);
         double *T = Tset + p.tens_off[v];
-        for (int64_t e = threadIdx.x; e < n; e += blockDim.x) {
-            int64_t r = e;
+        for (int e = rank * kWpThreads + tid; e < n; e += blocks * kWpThreads) {
+            int r = e;
             double w = 1.0;
             for (int i = k - 1; i >= 0; --i) {
-                const int dg = (int)(r % dims[i]);
-                r /= dims[i];
-                w *= sqrt(Sset[(int64_t)bonds[i] * kWpDim + dg]);
+                const int bd = p.site_bonds[l0 + i], dim = p.bond_dim[bd], dg = r % dim;
+                r /= dim;
+                w *= sqrt(__ldcg(Sset + (int64_t)bd * kWpDim + dg));
             }
-            T[e] *= w;
+            __stcg(T + e, __ldcg(T + e) * w);
         }
     }
+}
+
+template <int DM>
+cudaError_t launch_weight_passing(const WPParams &p, int blocks, cudaStream_t s)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(p.n_sets * blocks), 1, 1);
+    cfg.blockDim = dim3(kWpThreads, 1, 1);
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = (unsigned)blocks;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = blocks > 1 ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, weight_passing_kernel<DM>, p, blocks);
 }
 
 // ---------------------------------------------------------------- dense terms
@@ -776,11 +1035,20 @@ pne_status pne_weight_passing(pne_ctx *ctx, const pne_network *net, double alpha
     w->n_sets = B;
     const int64_t stride = g.tens_off[g.n_sites];
     int64_t tmax = 1;
+    int dmax = 1;
     for (int v = 0; v < g.n_sites; ++v) tmax = std::max<int64_t>(tmax, g.tens_off[v + 1] - g.tens_off[v]);
+    for (int b = 0; b < g.n_bonds; ++b) dmax = std::max(dmax, (int)g.bond_dim[b]);
+    // Blocks per set: two take the two sides of a bond, more share the rows of
+    // tensors above one panel, while every set's cluster fits the GPU at once.
+    // 3 x 3, chi = 16, 8 sets: 189, 124, 104 and 93 ms with 1, 2, 4 and 8 blocks;
+    // chi = 8 (512 rows): 64, 46.3, 45.7, 45.7.
+    int blocks = 1;
+    const int most = tmax / dmax > kWpPanel ? kWpCluster : 2;
+    while (2 * blocks <= most && 2 * blocks * B <= ctx->n_sm) blocks *= 2;
     DevBuf scratch, rec;
     if ((st = dev_alloc(ctx, w->T, (size_t)B * stride * 8, s)) ||
         (st = dev_alloc(ctx, w->S, (size_t)B * std::max(g.n_bonds, 1) * kWpDim * 8, s)) ||
-        (st = dev_alloc(ctx, scratch, (size_t)B * tmax * 8, s)) || (st = dev_alloc(ctx, rec, (size_t)B * 16, s))) {
+        (st = dev_alloc(ctx, scratch, (size_t)B * sizeof(WPShare), s)) || (st = dev_alloc(ctx, rec, (size_t)B * 16, s))) {
         dev_free(ctx, scratch, s); dev_free(ctx, rec, s); pne_weights_destroy(w);
         return st;
     }
@@ -791,14 +1059,17 @@ pne_status pne_weight_passing(pne_ctx *ctx, const pne_network *net, double alpha
     p.site_ptr = g.d_site_ptr; p.site_bonds = g.d_site_bonds; p.bond_dim = g.d_bond_dim; p.bond_site = g.d_bond_site;
     p.bond_leg = g.d_bond_leg; p.tens_off = g.d_tens_off; p.set_stride = stride;
     p.T = (double *)w->T.ptr; p.S = (double *)w->S.ptr;
-    p.scratch = (double *)scratch.ptr; p.scratch_per = tmax;
+    p.share = (WPShare *)scratch.ptr;
     p.alpha = alpha; p.tol = tol; p.max_sweeps = max_sweeps;
     p.log_scale = (double *)rec.ptr;
     p.sweeps = (int32_t *)((char *)rec.ptr + (size_t)B * 8);
     p.flags = p.sweeps + B;
     {
         ProfScope ps(ctx, s, "weight_passing");
-        weight_passing_kernel<<<B, kWpThreads, 0, s>>>(p);
+        const cudaError_t e = dmax <= 4   ? launch_weight_passing<4>(p, blocks, s)
+                              : dmax <= 8 ? launch_weight_passing<8>(p, blocks, s)
+                                          : launch_weight_passing<16>(p, blocks, s);
+        if (e != cudaSuccess) set_error(ctx, PNE_ECUDA, std::string("weight passing: ") + cudaGetErrorString(e));
     }
     PNE_LAUNCH_CHECK(ctx);
     std::vector<char> h((size_t)B * 16);
