@@ -27,10 +27,11 @@
 // a time in the same order, so their results are the same bit for bit.  The
 // grid's steps record the largest |entry| per set, from which the next step
 // takes a power-of-two scale (kept exactly in a log-2 counter).  The FP64 form
-// (f64_gemm_kernel) is a plain tiled GEMM on the CUDA cores with the same
-// interface: the reference the reduced-precision forms are stated against.
+// (f64_gemm_kernel) does the same products on the CUDA cores: the reference the
+// reduced-precision forms are stated against.
 #include <cuda.h>
 #include <cuda_runtime.h>
+#include <cooperative_groups.h>
 #include <cuda_bf16.h>
 #include <cudaTypedefs.h>
 
@@ -47,6 +48,7 @@
 #include "pne_internal.h"
 
 namespace pne {
+namespace cg = cooperative_groups;
 namespace {
 
 constexpr int kTcThreads = 128;
@@ -185,8 +187,7 @@ struct GemmParams {
     T *C;
     int64_t ldc, strideC;
     int M, N, K;
-    unsigned long long *maxbits;   // [batch]: largest |C| (bit pattern, atomicMax), or nullptr
-    int *err;                      // set to 1 when a bounded wait gave up
+    int *err;   // set to 1 when a bounded wait gave up
 };
 
 // 16 bytes of one row of a stage: EB = 4 -> 4 TF32 values, EB = 2 -> 8 BF16 values
@@ -295,7 +296,6 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc_gemm_kernel(GemmParams<float
         ok = __syncthreads_and(w) != 0;
     }
     tc_fence_after();
-    float mx = 0.f;
     const int row = m0 + warp * 32 + lane;
     if (ok) {
         for (int c0 = 0; c0 < BN; c0 += 16) {
@@ -305,169 +305,277 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc_gemm_kernel(GemmParams<float
                 float *dst = C + (int64_t)row * p.ldc + n0 + c0;
 #pragma unroll
                 for (int j = 0; j < 16; ++j) {
-                    const float v = __uint_as_float(r[j]);
-                    if (n0 + c0 + j < p.N) {
-                        dst[j] = v;
-                        mx = fmaxf(mx, fabsf(v));
-                    }
+                    if (n0 + c0 + j < p.N) dst[j] = __uint_as_float(r[j]);
                 }
             }
         }
     } else if (tid == 0) {
         atomicExch(p.err, 1);
     }
-    if (p.maxbits) {
-        for (int off = 16; off > 0; off >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, off));
-        if (lane == 0 && mx > 0.f) atomicMax(p.maxbits + set, (unsigned long long)__float_as_uint(mx));
-    }
     tc_fence_before();
     __syncthreads();
     if (warp == 0) tmem_dealloc(tmem, tcols);
 }
 
-// FP64 on the CUDA cores: 64 x 64 tile, 16-deep K slab, 4 x 4 outputs per thread
-constexpr int kF64Tile = 64, kF64Slab = 16;
+// ---------------------------------------------------------------- FP64 products
+// C = A B^T in FP64, and (RING) one site absorption of the grid contraction
+// with A read in the running tensor's ring order and scaled by 2^-e as the
+// tensor-core form does.  Bound by the FP64 pipes alone: a scheduler needs 64
+// clocks for one FP64 instruction of a warp, so the questions are how many of
+// its lanes do useful work, how evenly the instructions spread over the
+// schedulers, and that operand loads, which share the pipes' queue, are few.
+// The unit of work is 16 rows x 4 columns of C, two entries per lane (121
+// columns pad to 124), whose operands for two k are three 16-byte loads per
+// lane, two of them shared with the next unit of the same rows.  A block takes
+// a run of consecutive units of a block of up to 128 columns, its 16 warps (four
+// per scheduler) G units each, in registers; the host chooses the run so that
+// the SMs come out even.  64 x 64 tiles with 4 x 4 entries a thread, before,
+// padded 121 columns to 128 and left 458 tiles to 152 SMs: 15.1 ms for the 25
+// steps of a 5 x 5 grid of chi 11, now 11.0 (the FP64 pipes' own time 9.8 ms);
+// and gave 16 SMs work at M = N = K = 256: 305 us a call, now 72.
+// K goes in slabs, the next one copied while one is multiplied: of 32 where a
+// block has an SM to itself anyway, for fewer barriers, else of 16, so that two
+// fit.  Each entry is accumulated in the order of k.
+constexpr int kF64Threads = 512, kF64Warps = kF64Threads / 32;
+constexpr int kF64Rows = 256, kF64Cols = 128;            // staged rows of A and B
+constexpr int kF64MaxUnits = 12;                         // per warp
+constexpr int f64_slab(int G) { return G > 4 ? 32 : 16; }
+constexpr int f64_pitch(int G) { return f64_slab(G) + 2; }   // 16-byte loads of 8 rows on different banks
+constexpr int f64_stage(int G) { return (kF64Rows + kF64Cols) * f64_pitch(G); }
 
-__global__ void __launch_bounds__(256) f64_gemm_kernel(GemmParams<double> p)
+struct F64Params {
+    const double *A;
+    int64_t lda, strideA;
+    const double *B;
+    int64_t ldb, strideB;
+    double *C;
+    int64_t ldc, strideC;
+    int M, N, K;
+    int cub;                             // units (4 columns) per column block
+    int run;                             // units per block, <= kF64Warps * G
+    int64_t R;                           // RING: A[m][u Kh + h] = S[(u R + m) Kh + h]
+    int Kh;
+    const unsigned long long *max_in;    // [set] largest |S| (its bits)
+    unsigned long long *max_out;         // [set] largest |C|, atomicMax
+    unsigned long long *max_clear;       // [set] cleared for the next step
+    long long *log2s;                    // [set] += e
+};
+
+// 8 bytes into shared memory, zero when !ok (src is then not read)
+__device__ __forceinline__ void copy8_async(const double *dst, const double *src, bool ok)
 {
-    __shared__ double As[kF64Slab][kF64Tile + 1], Bs[kF64Slab][kF64Tile + 1];
-    const int set = blockIdx.z;
-    const int m0 = blockIdx.x * kF64Tile, n0 = blockIdx.y * kF64Tile;
+    const int n = ok ? 8 : 0;
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(smem_addr(dst)), "l"(src), "r"(n) : "memory");
+}
+
+template <int G, bool RING>
+__global__ void __launch_bounds__(kF64Threads, G > 4 ? 1 : 2) f64_gemm_kernel(F64Params p)
+{
+    constexpr int kSlab = f64_slab(G), kPitch = f64_pitch(G), kStage = f64_stage(G);
+    extern __shared__ __align__(16) double f64_smem[];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, set = blockIdx.z;
+    double sc = 1.0;
+    int e = 0;
+    if (RING) {
+        const double mx = __longlong_as_double((long long)p.max_in[set]);
+        if (mx > 0.0) e = ilogb(mx);
+        if (e) sc = ldexp(1.0, -e);
+        if (blockIdx.x == 0 && blockIdx.y == 0 && tid == 0) {
+            p.max_clear[set] = 0ull;
+            p.log2s[set] += e;
+        }
+    }
+    // the block's run of units (row group major) and the warp's part of it
+    const int c0 = blockIdx.y * p.cub, cub = min(p.cub, ((p.N - 1) >> 2) + 1 - c0);
+    const int64_t units = (int64_t)(((p.M - 1) >> 4) + 1) * cub, first = (int64_t)blockIdx.x * p.run;
+    if (first >= units) return;
+    const int run = (int)min((int64_t)p.run, units - first);
+    const int group0 = (int)(first / cub), skip = (int)(first - (int64_t)group0 * cub);
+    const int rows = 16 * ((skip + run - 1) / cub + 1);      // <= kF64Rows
+    const int cols = 4 * cub, m0 = 16 * group0, n0 = 4 * c0;
+    // warps w and w + 4 share a scheduler, so the odd units of a run go round them
+    const int share = run / kF64Warps, odd = run % kF64Warps;
+    const int u0 = skip + warp * share + min(warp, odd), g = share + (warp < odd ? 1 : 0);
+    const int r0 = u0 / cub, col0 = u0 - r0 * cub;
+    double acc[G][2];
+#pragma unroll
+    for (int i = 0; i < G; ++i) acc[i][0] = acc[i][1] = 0.0;
     const double *A = p.A + set * p.strideA, *B = p.B + set * p.strideB;
+    const int kk = tid & (kSlab - 1), row0 = tid / kSlab;
+    constexpr int kRowStep = kF64Threads / kSlab;
+    auto load = [&](int k0, double *st) {
+        const int k = k0 + kk;
+        int64_t a_off = k, a_row = p.lda;
+        if (RING) {
+            const int u = k / p.Kh;
+            a_off = (int64_t)u * p.R * p.Kh + (k - u * p.Kh);
+            a_row = p.Kh;
+        }
+        for (int r = row0; r < rows; r += kRowStep) {
+            const bool ok = k < p.K && m0 + r < p.M;
+            copy8_async(st + r * kPitch + kk, ok ? A + a_off + (m0 + r) * a_row : A, ok);
+        }
+        for (int r = row0; r < cols; r += kRowStep) {
+            const bool ok = k < p.K && n0 + r < p.N;
+            copy8_async(st + (kF64Rows + r) * kPitch + kk, ok ? B + (int64_t)(n0 + r) * p.ldb + k : B, ok);
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    load(0, f64_smem);
+    for (int k0 = 0, b = 0; k0 < p.K; k0 += kSlab, b ^= 1) {
+        double *st = f64_smem + b * kStage;
+        if (k0 + kSlab < p.K) {
+            load(k0 + kSlab, f64_smem + (b ^ 1) * kStage);
+            asm volatile("cp.async.wait_group 1;" ::: "memory");
+        } else {
+            asm volatile("cp.async.wait_group 0;" ::: "memory");
+        }
+        if (RING && e && k0 + kk < p.K) {                    // each thread the entries that it copied
+            for (int r = row0; r < rows; r += kRowStep) st[r * kPitch + kk] *= sc;
+        }
+        __syncthreads();
+        if (g > 0) {
+            const double *arow = st + (16 * r0 + (lane >> 2)) * kPitch;
+            const double *bcol = st + (kF64Rows + (lane & 3)) * kPitch;
+            const int kn = min(kSlab, p.K - k0);
+            for (int q = 0; q < kn; q += 2) {                // an odd K's last column is staged as zeros
+                const double *ar = arow + q;
+                int col = col0;
+                double2 a0 = *reinterpret_cast<const double2 *>(ar);
+                double2 a1 = *reinterpret_cast<const double2 *>(ar + 8 * kPitch);
+#pragma unroll
+                for (int i = 0; i < G; ++i) {
+                    if (i == G - 1 && i >= g) break;         // g is G or G - 1 but in a block's last run
+                    if (col == cub) {                        // the next row group
+                        col = 0;
+                        if (i < g) {
+                            ar += 16 * kPitch;
+                            a0 = *reinterpret_cast<const double2 *>(ar);
+                            a1 = *reinterpret_cast<const double2 *>(ar + 8 * kPitch);
+                        }
+                    }
+                    const double2 bv = *reinterpret_cast<const double2 *>(bcol + 4 * col * kPitch + q);
+                    acc[i][0] = fma(a0.x, bv.x, acc[i][0]);
+                    acc[i][1] = fma(a1.x, bv.x, acc[i][1]);
+                    acc[i][0] = fma(a0.y, bv.y, acc[i][0]);
+                    acc[i][1] = fma(a1.y, bv.y, acc[i][1]);
+                    ++col;
+                }
+            }
+        }
+        __syncthreads();
+    }
     double *C = p.C + set * p.strideC;
-    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-    double acc[4][4] = {};
-    for (int k0 = 0; k0 < p.K; k0 += kF64Slab) {
-        for (int i = threadIdx.x; i < kF64Slab * kF64Tile; i += blockDim.x) {
-            const int r = i / kF64Slab, kk = i % kF64Slab;
-            const int m = m0 + r, n = n0 + r, k = k0 + kk;
-            As[kk][r] = (m < p.M && k < p.K) ? A[(int64_t)m * p.lda + k] : 0.0;
-            Bs[kk][r] = (n < p.N && k < p.K) ? B[(int64_t)n * p.ldb + k] : 0.0;
-        }
-        __syncthreads();
+    unsigned long long mx = 0;
 #pragma unroll
-        for (int kk = 0; kk < kF64Slab; ++kk) {
-            double a[4], bv[4];
+    for (int i = 0; i < G; ++i) {
+        if (i >= g) continue;
+        const int r = (u0 + i) / cub;
+        const int m = m0 + 16 * r + (lane >> 2), n = n0 + 4 * (u0 + i - r * cub) + (lane & 3);
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                a[i] = As[kk][ty * 4 + i];
-                bv[i] = Bs[kk][tx * 4 + i];
-            }
-#pragma unroll
-            for (int i = 0; i < 4; ++i)
-#pragma unroll
-                for (int j = 0; j < 4; ++j) acc[i][j] = fma(a[i], bv[j], acc[i][j]);
-        }
-        __syncthreads();
-    }
-    double mx = 0.0;
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        const int m = m0 + ty * 4 + i;
-        if (m >= p.M) continue;
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const int n = n0 + tx * 4 + j;
-            if (n < p.N) {
-                C[(int64_t)m * p.ldc + n] = acc[i][j];
-                mx = fmax(mx, fabs(acc[i][j]));
+        for (int j = 0; j < 2; ++j) {
+            if (m + 8 * j >= p.M || n >= p.N) continue;
+            C[(int64_t)(m + 8 * j) * p.ldc + n] = acc[i][j];
+            if (RING) {                                      // largest |C| by its bits, a NaN passed over
+                const unsigned long long bits =
+                    (unsigned long long)__double_as_longlong(acc[i][j]) & 0x7fffffffffffffffull;
+                if (bits <= 0x7ff0000000000000ull && bits > mx) mx = bits;
             }
         }
     }
-    if (p.maxbits) {
-        for (int off = 16; off > 0; off >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, off));
-        if ((threadIdx.x & 31) == 0 && mx > 0.0)
-            atomicMax(p.maxbits + set, (unsigned long long)__double_as_longlong(mx));
+    if (RING) {
+        for (int off = 16; off > 0; off >>= 1) {
+            const unsigned long long o = __shfl_xor_sync(0xffffffffu, mx, off);
+            if (o > mx) mx = o;
+        }
+        if (lane == 0 && mx) atomicMax(p.max_out + set, mx);
     }
 }
 
 // ---------------------------------------------------------------- grid contraction
-// A[m][u Kh + h] = 2^-e * S[u][m][h], e the exponent of the set's largest |S|
-// (from maxbits[cur]); clears maxbits[next] and adds e to the set's log-2 scale.
-template <typename T>
-__global__ void grid_pack_kernel(const T *S, T *A, int64_t stride, int64_t R, int Ku, int Kh,
-                                 unsigned long long *maxbits_cur, unsigned long long *maxbits_next,
-                                 long long *log2s, int n_sets)
-{
-    const int set = blockIdx.y;
-    if (set >= n_sets) return;
-    const unsigned long long bits = maxbits_cur[set];
-    int e = 0;
-    if (sizeof(T) == 4) {
-        const float mx = __uint_as_float((unsigned)bits);
-        if (mx > 0.f) e = ilogbf(mx);
-    } else {
-        const double mx = __longlong_as_double((long long)bits);
-        if (mx > 0.0) e = ilogb(mx);
-    }
-    const T sc = (T)ldexp(1.0, -e);
-    const int K = Ku * Kh;
-    const int64_t total = R * K;
-    const T *s = S + set * stride;
-    T *a = A + set * stride;
-    for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < total; q += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t m = q / K;
-        const int k = (int)(q - m * K);
-        const int u = k / Kh, h = k - u * Kh;
-        a[q] = s[((int64_t)u * R + m) * Kh + h] * sc;
-    }
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-        maxbits_next[set] = 0ull;
-        log2s[set] += e;
-    }
-}
-
 // Site matrices B_v[n = d Nh + h'][k = u Kh + h] = 2^-s_v T_v[l = h, u, r = h', d]
-// per (set, site): one block, the largest |entry| first (s_v its exponent).
+// per (set, site), rows zero-padded to ldb, in the product's operand type; s_v
+// is the exponent of the tensor's largest |entry|.  A cluster of eight blocks
+// per tensor, each searching an eighth of it and writing an eighth of the rows,
+// a warp per row: at chi = 16 a tensor is 512 KB, and one block each with a
+// division per entry took 0.28 ms for 640 of them, this 0.12.
+constexpr int kSiteBlocks = 8;
 
-template <typename T>
-__global__ void grid_sites_kernel(const double *data, int64_t set_stride, const SiteMap *sites, int n_sites,
-                                  T *Bm, int64_t b_stride, long long *log2s)
+template <typename E>
+__device__ __forceinline__ E site_elem(double x);
+template <>
+__device__ __forceinline__ double site_elem<double>(double x) { return x; }
+template <>
+__device__ __forceinline__ float site_elem<float>(double x) { return __uint_as_float(to_tf32((float)x)); }
+template <>
+__device__ __forceinline__ __nv_bfloat16 site_elem<__nv_bfloat16>(double x) { return __float2bfloat16_rn((float)x); }
+
+template <typename E>
+__global__ void __cluster_dims__(1, 1, kSiteBlocks) __launch_bounds__(256)
+    grid_sites_kernel(const double *data, int64_t set_stride, const SiteMap *sites, E *Bm, int64_t b_stride,
+                      const int64_t *ldb, long long *log2s)
 {
-    const int v = blockIdx.x, set = blockIdx.y;
+    const int v = blockIdx.x, set = blockIdx.y, part = blockIdx.z;
     const SiteMap sm = sites[v];
     const double *t = data + set * set_stride + sm.t_off;
     const int Kh = sm.dim[0], Ku = sm.dim[1], Nh = sm.dim[2], Nd = sm.dim[3];
-    const int64_t n_ent = (int64_t)Kh * Ku * Nh * Nd;
-    __shared__ double red[32];
-    double mx = 0.0;
-    for (int64_t i = threadIdx.x; i < n_ent; i += blockDim.x) mx = fmax(mx, fabs(t[i]));
-    for (int off = 16; off > 0; off >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, off));
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = mx;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        for (int i = 1; i < (int)(blockDim.x >> 5); ++i) mx = fmax(mx, red[i]);
-        red[0] = mx;
-    }
-    __syncthreads();
-    mx = red[0];
-    const int e = mx > 0.0 ? ilogb(mx) : 0;
-    const double sc = ldexp(1.0, -e);
     const int K = Ku * Kh, N = Nd * Nh;
-    T *out = Bm + set * b_stride + sm.b_off;
-    for (int64_t q = threadIdx.x; q < (int64_t)N * K; q += blockDim.x) {
-        const int n = (int)(q / K), k = (int)(q % K);
-        const int d = n / Nh, hp = n % Nh, u = k / Kh, h = k % Kh;
-        const int64_t off = (int64_t)h * sm.stride[0] + (int64_t)u * sm.stride[1] + (int64_t)hp * sm.stride[2] +
-                            (int64_t)d * sm.stride[3];
-        out[q] = (T)(t[off] * sc);
+    const int64_t n_ent = (int64_t)N * K;
+    __shared__ unsigned long long largest[8];   // of each warp
+    cg::cluster_group cluster = cg::this_cluster();
+    // the largest |entry| by its bits (comparing doubles costs FP64 time), a NaN passed over
+    unsigned long long mx = 0;
+    for (int64_t i = part * 256 + threadIdx.x; i < n_ent; i += 256 * kSiteBlocks) {
+        const unsigned long long bits = (unsigned long long)__double_as_longlong(t[i]) & 0x7fffffffffffffffull;
+        if (bits <= 0x7ff0000000000000ull && bits > mx) mx = bits;
     }
-    if (threadIdx.x == 0) atomicAdd(reinterpret_cast<unsigned long long *>(log2s + set), (unsigned long long)(long long)e);
+    for (int off = 16; off > 0; off >>= 1) {
+        const unsigned long long o = __shfl_xor_sync(0xffffffffu, mx, off);
+        if (o > mx) mx = o;
+    }
+    if ((threadIdx.x & 31) == 0) largest[threadIdx.x >> 5] = mx;
+    cluster.sync();
+    mx = 0;
+    for (int i = threadIdx.x & 31; i < 8 * kSiteBlocks; i += 32) {
+        const unsigned long long o = cluster.map_shared_rank(largest, i >> 3)[i & 7];
+        if (o > mx) mx = o;
+    }
+    for (int off = 16; off > 0; off >>= 1) {
+        const unsigned long long o = __shfl_xor_sync(0xffffffffu, mx, off);
+        if (o > mx) mx = o;
+    }
+    cluster.sync();                             // no block leaves while its maxima are read
+    const double top = __longlong_as_double((long long)mx);
+    const int e = top > 0.0 ? ilogb(top) : 0;
+    const double sc = ldexp(1.0, -e);
+    const int ld = (int)ldb[v];
+    E *out = Bm + set * b_stride + sm.b_off;
+    for (int n = part * 8 + (threadIdx.x >> 5); n < N; n += 8 * kSiteBlocks) {
+        const int d = n / Nh, hp = n - d * Nh;
+        const double *row = t + (int64_t)hp * sm.stride[2] + (int64_t)d * sm.stride[3];
+        for (int k = threadIdx.x & 31; k < ld; k += 32) {
+            const int u = k / Kh, h = k - u * Kh;
+            out[(int64_t)n * ld + k] =
+                site_elem<E>(k < K ? row[(int64_t)h * sm.stride[0] + (int64_t)u * sm.stride[1]] * sc : 0.0);
+        }
+    }
+    if (part == 0 && threadIdx.x == 0)
+        atomicAdd(reinterpret_cast<unsigned long long *>(log2s + set), (unsigned long long)(long long)e);
 }
 
-template <typename T>
-__global__ void grid_init_kernel(T *S, int64_t stride, unsigned long long *maxbits, long long *log2s, int n_sets)
+template <typename E>
+__global__ void grid_init_kernel(E *S, int64_t stride, unsigned long long *maxbits, long long *log2s, int n_sets)
 {
     const int set = blockIdx.x * blockDim.x + threadIdx.x;
     if (set >= n_sets) return;
-    S[set * stride] = (T)1;
-    maxbits[set] = sizeof(T) == 4 ? (unsigned long long)__float_as_uint(1.0f)
-                                  : (unsigned long long)__double_as_longlong(1.0);
+    S[set * stride] = site_elem<E>(1.0);
+    maxbits[set] = sizeof(E) == 8 ? (unsigned long long)__double_as_longlong(1.0)
+                                  : (unsigned long long)__float_as_uint(1.0f);
     log2s[set] = 0;
 }
 
-template <typename T>
-__global__ void grid_final_kernel(const T *S, int64_t stride, const long long *log2s, int n_sets, double *out)
+template <typename E>
+__global__ void grid_final_kernel(const E *S, int64_t stride, const long long *log2s, int n_sets, double *out)
 {
     const int set = blockIdx.x * blockDim.x + threadIdx.x;
     if (set >= n_sets) return;
@@ -497,83 +605,6 @@ struct RingParams {
     long long *log2s;                   // [set] += e_in
     int *err;
 };
-
-template <typename E>
-__device__ __forceinline__ float elem_to_float(E x);
-template <>
-__device__ __forceinline__ float elem_to_float<float>(float x) { return x; }
-template <>
-__device__ __forceinline__ float elem_to_float<__nv_bfloat16>(__nv_bfloat16 x) { return __bfloat162float(x); }
-
-template <typename E>
-__device__ __forceinline__ E round_elem(float x);
-template <>
-__device__ __forceinline__ float round_elem<float>(float x) { return __uint_as_float(to_tf32(x)); }
-template <>
-__device__ __forceinline__ __nv_bfloat16 round_elem<__nv_bfloat16>(float x) { return __float2bfloat16_rn(x); }
-
-// Site matrices for the tensor-core path: rows padded to a multiple of the
-// 16-byte unit, entries scaled by 2^-s_v and rounded to the operand type.
-template <typename E>
-__global__ void grid_sites_tc_kernel(const double *data, int64_t set_stride, const SiteMap *sites, E *Bm,
-                                     int64_t b_stride, const int64_t *ldb, long long *log2s)
-{
-    const int v = blockIdx.x, set = blockIdx.y;
-    const SiteMap sm = sites[v];
-    const double *t = data + set * set_stride + sm.t_off;
-    const int Kh = sm.dim[0], Ku = sm.dim[1], Nh = sm.dim[2], Nd = sm.dim[3];
-    const int64_t n_ent = (int64_t)Kh * Ku * Nh * Nd;
-    __shared__ double red[32];
-    double mx = 0.0;
-    for (int64_t i = threadIdx.x; i < n_ent; i += blockDim.x) mx = fmax(mx, fabs(t[i]));
-    for (int off = 16; off > 0; off >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, off));
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = mx;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        for (int i = 1; i < (int)(blockDim.x >> 5); ++i) mx = fmax(mx, red[i]);
-        red[0] = mx;
-    }
-    __syncthreads();
-    mx = red[0];
-    const int e = mx > 0.0 ? ilogb(mx) : 0;
-    const double sc = ldexp(1.0, -e);
-    const int K = Ku * Kh, N = Nd * Nh;
-    const int64_t ld = ldb[v];
-    E *out = Bm + set * b_stride + sm.b_off;
-    for (int64_t q = threadIdx.x; q < (int64_t)N * ld; q += blockDim.x) {
-        const int n = (int)(q / ld), k = (int)(q % ld);
-        float x = 0.f;
-        if (k < K) {
-            const int d = n / Nh, hp = n % Nh, u = k / Kh, h = k % Kh;
-            const int64_t off = (int64_t)h * sm.stride[0] + (int64_t)u * sm.stride[1] + (int64_t)hp * sm.stride[2] +
-                                (int64_t)d * sm.stride[3];
-            x = (float)(t[off] * sc);
-        }
-        out[q] = round_elem<E>(x);
-    }
-    if (threadIdx.x == 0) atomicAdd(reinterpret_cast<unsigned long long *>(log2s + set), (unsigned long long)(long long)e);
-}
-
-template <typename E>
-__global__ void grid_init_tc_kernel(E *S, int64_t stride, unsigned long long *maxbits, long long *log2s, int n_sets)
-{
-    const int set = blockIdx.x * blockDim.x + threadIdx.x;
-    if (set >= n_sets) return;
-    S[set * stride] = round_elem<E>(1.f);
-    maxbits[set] = (unsigned long long)__float_as_uint(1.0f);
-    log2s[set] = 0;
-}
-
-template <typename E>
-__global__ void grid_final_tc_kernel(const E *S, int64_t stride, const unsigned long long *max_last,
-                                     const long long *log2s, int n_sets, double *out)
-{
-    const int set = blockIdx.x * blockDim.x + threadIdx.x;
-    if (set >= n_sets) return;
-    out[2 * set] = (double)elem_to_float<E>(S[set * stride]);
-    out[2 * set + 1] = (double)log2s[set];
-    (void)max_last;
-}
 
 // ---------------------------------------------------------------- the persistent GEMM
 // One kernel for the large products, by where A comes from:
@@ -1240,12 +1271,59 @@ cudaError_t launch_tc(pne_ctx *ctx, const GemmParams<float> &p, int batch, cudaS
     return cudaGetLastError();
 }
 
-cudaError_t launch_f64(const GemmParams<double> &p, int batch, cudaStream_t s)
+template <int G, bool RING>
+cudaError_t launch_f64_units(const F64Params &p, dim3 grid, cudaStream_t s)
 {
-    const dim3 grid((unsigned)((p.M + kF64Tile - 1) / kF64Tile), (unsigned)((p.N + kF64Tile - 1) / kF64Tile),
-                    (unsigned)batch);
-    f64_gemm_kernel<<<grid, 256, 0, s>>>(p);
+    const size_t smem = 2 * f64_stage(G) * sizeof(double);
+    const cudaError_t e = grant_dynamic_smem((const void *)f64_gemm_kernel<G, RING>, smem);
+    if (e != cudaSuccess) return e;
+    f64_gemm_kernel<G, RING><<<grid, kF64Threads, smem, s>>>(p);
     return cudaGetLastError();
+}
+
+// A block's run of f64_gemm_kernel: for the fewest waves of one block per SM that
+// 12 units a warp allow, and three more, as many blocks as the waves hold; of
+// these the run that ends first, a wave taking its units per scheduler and two
+// more for filling and storing; or four units a warp, whose blocks share an SM
+// by twos and so hide that (M = N = 4096, K = 512, 13.7 ms on the pipes alone:
+// 13.88 ms, 14.15 as waves of single blocks).  A run of n units may touch
+// (n - 2) / columns + 2 row groups, of which 16 are staged, so few columns take
+// short runs; four units are one per scheduler.
+template <bool RING>
+cudaError_t launch_f64(F64Params p, int batch, int n_sm, cudaStream_t s)
+{
+    const int64_t groups = (p.M - 1) / 16 + 1, cu = (p.N - 1) / 4 + 1;
+    const int64_t cblocks = (cu + kF64Cols / 4 - 1) / (kF64Cols / 4);
+    p.cub = (int)((cu + cblocks - 1) / cblocks);
+    const int64_t units = groups * p.cub, P = cblocks * batch;
+    const int64_t narrow = cu - (cblocks - 1) * p.cub;       // units across the last column block
+    const int64_t most = std::min<int64_t>(kF64Warps * kF64MaxUnits, (kF64Rows / 16 - 1) * narrow + 1);
+    const int64_t least = (units + most - 1) / most, w0 = (P * least + n_sm - 1) / n_sm;
+    int64_t cost = INT64_MAX;
+    for (int64_t w = w0; w < w0 + 4; ++w) {
+        const int64_t b = w * n_sm / P;
+        const int64_t run = std::max<int64_t>((units + b - 1) / b, 4);
+        if (w * ((run + 3) / 4 + 2) >= cost) continue;
+        cost = w * ((run + 3) / 4 + 2);
+        p.run = (int)run;
+    }
+    const int64_t pair = std::min<int64_t>(kF64Warps * 4, most);
+    if (((units + pair - 1) / pair * P + n_sm - 1) / n_sm * ((pair + 3) / 4) + 2 < cost) p.run = (int)pair;
+    const dim3 grid((unsigned)((units + p.run - 1) / p.run), (unsigned)cblocks, (unsigned)batch);
+    switch ((p.run + kF64Warps - 1) / kF64Warps) {
+    case 1: return launch_f64_units<1, RING>(p, grid, s);
+    case 2: return launch_f64_units<2, RING>(p, grid, s);
+    case 3: return launch_f64_units<3, RING>(p, grid, s);
+    case 4: return launch_f64_units<4, RING>(p, grid, s);
+    case 5: return launch_f64_units<5, RING>(p, grid, s);
+    case 6: return launch_f64_units<6, RING>(p, grid, s);
+    case 7: return launch_f64_units<7, RING>(p, grid, s);
+    case 8: return launch_f64_units<8, RING>(p, grid, s);
+    case 9: return launch_f64_units<9, RING>(p, grid, s);
+    case 10: return launch_f64_units<10, RING>(p, grid, s);
+    case 11: return launch_f64_units<11, RING>(p, grid, s);
+    default: return launch_f64_units<kF64MaxUnits, RING>(p, grid, s);
+    }
 }
 
 }  // namespace
@@ -1378,9 +1456,9 @@ pne_status grid_run(pne_ctx *ctx, const GridPlan &plan, const double *data, int6
             E *S0 = (E *)dS.ptr, *S1 = (E *)dA.ptr;
             {
                 ProfScope ps(ctx, s, "grid_sites");
-                grid_init_tc_kernel<E><<<ib, 128, 0, s>>>(S0, max_state, mb, lg, nb);
-                grid_sites_tc_kernel<E><<<dim3(n, nb), 256, 0, s>>>(data, set_stride, (const SiteMap *)dMaps.ptr,
-                                                                    (E *)dB.ptr, b_total, (const int64_t *)dLdb.ptr, lg);
+                grid_init_kernel<E><<<ib, 128, 0, s>>>(S0, max_state, mb, lg, nb);
+                grid_sites_kernel<E><<<dim3(n, nb, kSiteBlocks), 256, 0, s>>>(
+                    data, set_stride, (const SiteMap *)dMaps.ptr, (E *)dB.ptr, b_total, (const int64_t *)dLdb.ptr, lg);
             }
             cudaError_t ee = cudaGetLastError();
             if (ee != cudaSuccess) return ee;
@@ -1409,46 +1487,51 @@ pne_status grid_run(pne_ctx *ctx, const GridPlan &plan, const double *data, int6
             }
             {
                 ProfScope ps(ctx, s, "grid_final");
-                grid_final_tc_kernel<E><<<ib, 128, 0, s>>>((n & 1) ? S1 : S0, max_state, mb, lg, nb, (double *)dOut.ptr);
+                grid_final_kernel<E><<<ib, 128, 0, s>>>((n & 1) ? S1 : S0, max_state, lg, nb, (double *)dOut.ptr);
             }
             return cudaGetLastError();
         };
         e = dtype == PNE_TF32 ? run_tc(float(0)) : run_tc(__nv_bfloat16());
         if (e != cudaSuccess) return fail(e, "grid contraction (tensor cores)");
     } else {
+        double *S0 = (double *)dS.ptr, *S1 = (double *)dA.ptr;
         {
             ProfScope ps(ctx, s, "grid_sites");
-            grid_init_kernel<double><<<ib, 128, 0, s>>>((double *)dS.ptr, max_state, mb, lg, nb);
-            grid_sites_kernel<double><<<dim3(n, nb), 256, 0, s>>>(data, set_stride, (const SiteMap *)dMaps.ptr, n,
-                                                                  (double *)dB.ptr, b_total, lg);
+            grid_init_kernel<double><<<ib, 128, 0, s>>>(S0, max_state, mb, lg, nb);
+            grid_sites_kernel<double><<<dim3(n, nb, kSiteBlocks), 256, 0, s>>>(
+                data, set_stride, (const SiteMap *)dMaps.ptr, (double *)dB.ptr, b_total, (const int64_t *)dLdb.ptr, lg);
         }
         if ((e = cudaGetLastError()) != cudaSuccess) return fail(e, "grid site matrices");
         for (int v = 0; v < n; ++v) {
             const GridStep &sd = plan.steps[(size_t)v];
-            const int K = sd.Ku * sd.Kh, N = sd.Nd * sd.Nh;
-            unsigned long long *cur = mb + (size_t)(v & 1) * nb, *nxt = mb + (size_t)((v + 1) & 1) * nb;
-            const int64_t total = sd.R * K;
-            const int pblocks = (int)std::min<int64_t>((total + 255) / 256, 152 * 8);
-            {
-                ProfScope ps(ctx, s, "grid_pack");
-                grid_pack_kernel<double><<<dim3(pblocks, nb), 256, 0, s>>>((const double *)dS.ptr, (double *)dA.ptr,
-                                                                          max_state, sd.R, sd.Ku, sd.Kh, cur, nxt, lg,
-                                                                          nb);
-            }
-            if ((e = cudaGetLastError()) != cudaSuccess) return fail(e, "grid_pack_kernel");
+            F64Params p{};
+            p.A = (v & 1) ? S1 : S0;
+            p.strideA = max_state;
+            p.B = (const double *)dB.ptr + plan.maps[(size_t)v].b_off;
+            p.ldb = plan.ldb[(size_t)v];
+            p.strideB = b_total;
+            p.C = (v & 1) ? S0 : S1;
+            p.strideC = max_state;
+            p.M = (int)sd.R;
+            p.N = sd.Nd * sd.Nh;
+            p.K = sd.Ku * sd.Kh;
+            p.ldc = p.N;
+            p.R = sd.R;
+            p.Kh = sd.Kh;
+            p.max_in = mb + (size_t)(v % 3) * nb;
+            p.max_out = mb + (size_t)((v + 1) % 3) * nb;
+            p.max_clear = mb + (size_t)((v + 2) % 3) * nb;
+            p.log2s = lg;
             {
                 ProfScope ps(ctx, s, "grid_gemm_f64");
-                GemmParams<double> p{(const double *)dA.ptr, K, max_state,
-                                     (const double *)dB.ptr + plan.maps[(size_t)v].b_off, K, b_total,
-                                     (double *)dS.ptr, N, max_state, (int)sd.R, N, K, nxt, (int *)dErr.ptr};
-                e = launch_f64(p, nb, s);
+                e = launch_f64<true>(p, nb, ctx->n_sm, s);
             }
             if (e != cudaSuccess) return fail(e, "grid GEMM");
-            bound += (double)K * std::ldexp(1.0, -53);
+            bound += (double)p.K * std::ldexp(1.0, -53);
         }
         {
             ProfScope ps(ctx, s, "grid_final");
-            grid_final_kernel<double><<<ib, 128, 0, s>>>((const double *)dS.ptr, max_state, lg, nb, (double *)dOut.ptr);
+            grid_final_kernel<double><<<ib, 128, 0, s>>>((n & 1) ? S1 : S0, max_state, lg, nb, (double *)dOut.ptr);
         }
         if ((e = cudaGetLastError()) != cudaSuccess) return fail(e, "grid_final_kernel");
     }
@@ -1490,12 +1573,23 @@ pne_status pne_dense_gemm(pne_ctx *ctx, pne_dtype dtype, int32_t batch, int32_t 
     if (e == cudaSuccess) {
         ProfScope ps(ctx, s, dtype == PNE_F64 ? "dense_gemm_f64" : "dense_gemm_tc");
         if (dtype == PNE_F64) {
-            GemmParams<double> p{(const double *)A, lda, strideA, (const double *)B, ldb, strideB, (double *)C, ldc,
-                                 strideC, M, N, K, nullptr, (int *)err.ptr};
-            e = launch_f64(p, batch, s);
+            F64Params p{};
+            p.A = (const double *)A;
+            p.lda = lda;
+            p.strideA = strideA;
+            p.B = (const double *)B;
+            p.ldb = ldb;
+            p.strideB = strideB;
+            p.C = (double *)C;
+            p.ldc = ldc;
+            p.strideC = strideC;
+            p.M = M;
+            p.N = N;
+            p.K = K;
+            e = launch_f64<false>(p, batch, ctx->n_sm, s);
         } else {
             GemmParams<float> p{(const float *)A, lda, strideA, (const float *)B, ldb, strideB, (float *)C, ldc,
-                                strideC, M, N, K, nullptr, (int *)err.ptr};
+                                strideC, M, N, K, (int *)err.ptr};
             e = dtype == PNE_TF32 ? launch_tc<4>(ctx, p, batch, s) : launch_tc<2>(ctx, p, batch, s);
         }
     }
