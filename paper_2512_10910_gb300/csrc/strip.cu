@@ -43,6 +43,7 @@ namespace {
 constexpr int kMaxL = PNE_STRIP_MAX_L;
 constexpr int kMaxChi = PNE_STRIP_MAX_CHI;
 constexpr int kThreads = 256;
+constexpr int kApplyThreads = 128;              // short blocks: fewer SMs wait for the last ones
 constexpr int kRedBlocks = 512;                 // reduction blocks per tensor
 constexpr int64_t kMaxState = (int64_t)1 << 28; // chi^(L+1) limit (2 GiB of doubles)
 constexpr double kGroupBytes = 24e9;            // working set of one group of tensors
@@ -239,11 +240,20 @@ struct ApplyParams {
 
 // out[p][o][s] = sum_i mat[o][i] * in[p][i][s] (* scale): one site of the row.
 // IN / OUT formats: 0 FP64, 1 float-float pair (hi, lo) in the same 8 bytes.
-// With FF the multiply-adds run on the FP32 pipes as compensated dot products
-// (each product split exactly by one FMA, the running sum by Knuth's two-sum,
-// the error terms and the low-part cross products gathered in one FP32
-// compensation): about 2^-48 relative to sum |a x| per output, where the FP64
-// pipe of this part retires 1/60 of the FP32 rate.
+// With FF the multiply-adds run on the FP32 pipes as compensated dot products:
+// the running sum by Knuth's two-sum, whose second difference is taken from
+// the unrounded product by an FMA and so carries the product's own rounding
+// too, the error terms and the low-part cross products gathered in one FP32
+// compensation: about 2^-48 relative to sum |a x| per output, where the FP64
+// pipe of this part retires 1/60 of the FP32 rate.  That is ten instructions a
+// multiply-add; with the product split by an FMA of its own it was twelve, and
+// no more exact.  The FP32 pipes bound it (63% busy, 72% of the issue slots: the
+// rest is lost to operand conflicts), so the matrix comes in 16-byte loads of
+// two entries' pairs and an index costs one 32-bit division.  Row products of a
+// call, ms before and now: chi 4, 7 wide, 8 tensors 7.2, 5.6; 10 wide 86, 77;
+// chi 5, 8 wide, 2 tensors 17.8, 13.5; chi 8, 6 wide, 2 tensors 26.2, 17.6.
+// Packed FP32 instructions (two fibres a thread) were slower, 82 ms at chi 4,
+// 10 wide, and so was taking few enough tensors at a time to stay in L2 (88).
 struct ffp { float h, l; };
 
 __device__ __forceinline__ ffp split_double(double x)
@@ -253,19 +263,19 @@ __device__ __forceinline__ ffp split_double(double x)
 }
 
 template <int NIN, int NOUT, int IN_FF, int OUT_FF>
-__global__ void __launch_bounds__(kThreads) strip_apply_kernel(ApplyParams p)
+__global__ void __launch_bounds__(kApplyThreads) strip_apply_kernel(ApplyParams p)
 {
     const int b = blockIdx.y;
     if (p.st[b].done) return;
     constexpr bool FF = IN_FF || OUT_FF;
+    constexpr int kPairs = (NIN + 1) / 2;                    // a row of M as (high, low) pairs, two to a load
     __shared__ double M[FF ? 1 : NOUT * NIN];
-    __shared__ float Mh[FF ? NOUT * NIN : 1], Ml[FF ? NOUT * NIN : 1];
+    __shared__ float4 Mf[FF ? NOUT * kPairs : 1];
     const double *mat = p.ops + b * p.ops_stride + p.mat_off;
     for (int i = threadIdx.x; i < NOUT * NIN; i += blockDim.x) {
         if (FF) {
             const ffp a = split_double(mat[i]);
-            Mh[i] = a.h;
-            Ml[i] = a.l;
+            reinterpret_cast<float2 *>(Mf + i / NIN * kPairs)[i % NIN] = make_float2(a.h, a.l);
         } else {
             M[i] = mat[i];
         }
@@ -274,7 +284,7 @@ __global__ void __launch_bounds__(kThreads) strip_apply_kernel(ApplyParams p)
     const double sc = p.use_scale ? p.st[b].scale : 1.0;
     const int64_t units = p.P * p.S;
     for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < units; q += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t pp = q / p.S, s = q - pp * p.S;
+        const int64_t pp = (uint32_t)q / (uint32_t)p.S, s = q - pp * p.S;    // units <= kMaxState
         const int64_t src0 = (pp * NIN) * p.S + s, dst0 = (pp * NOUT) * p.S + s;
         if (!FF) {
             const double *in = p.in + b * p.in_stride + src0;
@@ -313,14 +323,19 @@ __global__ void __launch_bounds__(kThreads) strip_apply_kernel(ApplyParams p)
                 float sh = 0.f, c = 0.f;
 #pragma unroll
                 for (int i = 0; i < NIN; ++i) {
-                    const float ah = Mh[o * NIN + i], al = Ml[o * NIN + i];
+                    const float4 m = Mf[o * kPairs + i / 2];
+                    const float ah = i & 1 ? m.z : m.x, al = i & 1 ? m.w : m.y;
                     const float pr = __fmul_rn(ah, xh[i]);
-                    const float e = __fmaf_rn(ah, xh[i], -pr);
-                    const float t = __fadd_rn(sh, pr);
-                    const float bb = __fsub_rn(t, sh);
-                    const float q2 = __fadd_rn(__fsub_rn(sh, __fsub_rn(t, bb)), __fsub_rn(pr, bb));
-                    sh = t;
-                    c = __fadd_rn(c, __fadd_rn(q2, e));
+                    if (i == 0) {
+                        sh = pr;
+                        c = __fmaf_rn(ah, xh[i], -pr);
+                    } else {
+                        const float t = __fadd_rn(sh, pr);
+                        const float bb = __fsub_rn(t, sh);
+                        const float e = __fmaf_rn(ah, xh[i], -bb);   // the product's share of t's error, and its own
+                        c = __fadd_rn(c, __fadd_rn(__fsub_rn(sh, __fsub_rn(t, bb)), e));
+                        sh = t;
+                    }
                     c = __fmaf_rn(ah, xl[i], c);
                     c = __fmaf_rn(al, xh[i], c);
                 }
@@ -347,11 +362,11 @@ __global__ void strip_init_kernel(double *V, int64_t stride, const double *ops, 
     const double *top = ops + b * ops_stride + top_off;
     double *v = V + b * stride;
     for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < N; q += (int64_t)gridDim.x * blockDim.x) {
-        int64_t r = q;
+        uint32_t r = (uint32_t)q;                            // N <= kMaxState
         double x = 1.0;
         for (int i = 0; i < k; ++i) {
-            x *= top[r % chi];
-            r /= chi;
+            x *= top[r % (uint32_t)chi];
+            r /= (uint32_t)chi;
         }
         v[q] = x;
     }
@@ -445,12 +460,12 @@ __global__ void __launch_bounds__(kThreads) strip_reduce_kernel(const double *V,
         const double x = w[q];
         ww = fma(x, x, ww);
         vw = fma(v[q], x, vw);
-        int64_t t = q;
-        double c = r ? tabP[t % cr] : 1.0;
-        if (r) t /= cr;
+        uint32_t t = (uint32_t)q, rest = t / (uint32_t)cr;   // N <= kMaxState
+        double c = tabP[t - rest * cr];
         for (int i = 0; i < ng; ++i) {
-            c *= tabF[t % cg];
-            t /= cg;
+            t = rest;
+            rest = t / (uint32_t)cg;
+            c *= tabF[t - rest * cg];
         }
         wc = fma(x, c, wc);
     }
@@ -697,9 +712,9 @@ template <int NIN, int NOUT, int IN_FF, int OUT_FF>
 cudaError_t launch_apply(const ApplyParams &p, int n, cudaStream_t s)
 {
     const int64_t units = p.P * p.S;
-    int64_t blocks = (units + kThreads - 1) / kThreads;
-    blocks = std::min<int64_t>(std::max<int64_t>(blocks, 1), 152 * 16);
-    strip_apply_kernel<NIN, NOUT, IN_FF, OUT_FF><<<dim3((unsigned)blocks, (unsigned)n), kThreads, 0, s>>>(p);
+    int64_t blocks = (units + kApplyThreads - 1) / kApplyThreads;
+    blocks = std::min<int64_t>(std::max<int64_t>(blocks, 1), 152 * 32);
+    strip_apply_kernel<NIN, NOUT, IN_FF, OUT_FF><<<dim3((unsigned)blocks, (unsigned)n), kApplyThreads, 0, s>>>(p);
     return cudaGetLastError();
 }
 
