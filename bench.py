@@ -746,7 +746,7 @@ def run_strip_extra(args, ctx, pne, torch, dev, local_rank):
             pne.pne_ctx_profile(ctx.h, False)
             flops = sum(r["iters"][o][k] * _strip_row_flops(4, k) for r in res for o in (0, 1) for k in range(1, L + 1))
             row_ms = prof.get("strip_row", (0, 0.0))[1]
-            peak = peak64 if arith == 0 else peak32 / 12.0
+            peak = peak64 if arith == 0 else peak32 / 10.0
             rec = {"wall_s": wall, "kernel_ms": {k: round(v[1], 3) for k, v in prof.items()},
                    "max_rel_err_vs_onsager": max(abs(r["f"] - exact[i]) / abs(exact[i]) for i, r in zip(sel, res)),
                    "rel_err_by_beta": {f"{betas[i]:.2f}": abs(r["f"] - exact[i]) / abs(exact[i])
@@ -760,7 +760,7 @@ def run_strip_extra(args, ctx, pne, torch, dev, local_rank):
                                     "work": "2 flops per multiply-add of the site-by-site row products, summed over "
                                             "every power iteration of every width and orientation",
                                     "peak_source": ("measured FP64 FMA-chain kernel" if arith == 0 else
-                                                    "measured FP32 FMA-chain kernel / 12 FP32 instructions per "
+                                                    "measured FP32 FMA-chain kernel / 10 FP32 instructions per "
                                                     "float-float multiply-add")}}
             out[f"{tag}_{aname}"] = rec
     return out
