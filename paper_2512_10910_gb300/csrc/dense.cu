@@ -938,7 +938,17 @@ __global__ void __launch_bounds__(stream_threads(SRC), 1) tc_stream_kernel(const
                 uint8_t *dst = out + ((m0 + row1) * p.ldc + col) * OB;
                 const int64_t hop = 4 * p.ldc * OB;
                 const int rows = (int)min((int64_t)32, p.M - m0);
-                if (p.vec && left >= EPO) {
+                if (RAW && !p.vec) {                            // unaligned rows of FP32: a line of one row at a time
+                    const int cc = n * p.BN + c0 + lane;
+                    const bool in = cc < min(p.N, (n + 1) * p.BN);
+                    uint32_t *line = reinterpret_cast<uint32_t *>(out) + m0 * p.ldc + cc;
+#pragma unroll 8
+                    for (int rr = 0; rr < 32; ++rr) {
+                        const uint32_t v = *reinterpret_cast<const uint32_t *>(
+                            buf + rr * 128 + (((lane >> 2) ^ (rr & 7)) * 16) + (lane & 3) * 4);
+                        if (in && rr < rows) line[rr * p.ldc] = v;
+                    }
+                } else if (p.vec && left >= EPO) {
 #pragma unroll
                     for (int i = 0; i < 8; ++i) {
                         const int rr = i * 4 + row1;
@@ -1237,6 +1247,53 @@ cudaError_t launch_dense_stream(const GemmParams<float> &p, int batch, int n_sm,
     return e != cudaSuccess ? e : launch_stream<EB, kRound>(ma, mb, q, n_sm, s);
 }
 
+// Rows of A that the copy engine cannot address, one warp per row, to rows of
+// ldp values (a multiple of four; the padding is never read)
+__global__ void pad_rows_kernel(const float *A, int64_t lda, int64_t strideA, int M, int K, int64_t rows, int64_t ldp,
+                                float *P)
+{
+    const int lane = threadIdx.x & 31;
+    for (int64_t r = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); r < rows;
+         r += (int64_t)gridDim.x * (blockDim.x >> 5)) {
+        const int64_t b = r / M;
+        const float *src = A + b * strideA + (r - b * M) * lda;
+        float *dst = P + r * ldp;
+#pragma unroll 4
+        for (int k = lane; k < K; k += 32) dst[k] = __ldg(src + k);
+    }
+}
+
+// The persistent kernel behind a padded copy of A, a piece of at most kPadBytes
+// at a time: several whole sets, or a range of one set's rows.
+constexpr int64_t kPadBytes = (int64_t)96 << 20;
+
+template <int EB>
+cudaError_t launch_padded_stream(const GemmParams<float> &p, int batch, int n_sm, float *P, int64_t ldp, void *W,
+                                 int64_t ldw, cudaStream_t s, bool &used)
+{
+    const int64_t most = std::max<int64_t>(kPadBytes / (ldp * 4) / kTcBM * kTcBM, kTcBM);
+    const int sets = (int)std::min<int64_t>(batch, std::max<int64_t>(1, most / p.M));
+    const int64_t rows = std::min<int64_t>(p.M, most);
+    for (int b = 0; b < batch; b += sets)
+        for (int64_t m = 0; m < p.M; m += rows) {
+            const int nb = std::min(sets, batch - b);
+            GemmParams<float> q = p;
+            q.M = (int)std::min<int64_t>(rows, p.M - m);
+            q.A = P;
+            q.lda = ldp;
+            q.strideA = ldp * q.M;
+            q.B = p.B + b * p.strideB;
+            q.C = p.C + b * p.strideC + m * p.ldc;
+            const int64_t n = (int64_t)nb * q.M;
+            pad_rows_kernel<<<(unsigned)std::min<int64_t>((n + 7) / 8, (int64_t)n_sm * 16), 256, 0, s>>>(
+                p.A + b * p.strideA + m * p.lda, p.lda, p.strideA, q.M, p.K, n, ldp, P);
+            cudaError_t e = cudaGetLastError();
+            if (e == cudaSuccess) e = launch_dense_stream<EB>(q, nb, n_sm, W, ldw, s, used);
+            if (e != cudaSuccess || !used) return e;
+        }
+    return cudaSuccess;
+}
+
 template <int EB>
 cudaError_t launch_tc(pne_ctx *ctx, const GemmParams<float> &p, int batch, cudaStream_t s)
 {
@@ -1250,13 +1307,24 @@ cudaError_t launch_tc(pne_ctx *ctx, const GemmParams<float> &p, int batch, cudaS
     // the later (16 x 640 x 64 x 100: 45.9 against 36.2 TF32, 34.6 against 35.8
     // BF16); many blocks take it at any K.
     const int64_t blocks = (int64_t)((p.M + kTcBM - 1) / kTcBM) * ((p.N + BN - 1) / BN) * batch;
-    const bool large = (int64_t)p.K * (kTcBM + BN) >= (EB == 4 ? 14000 : 20000) || blocks >= 2 * ctx->n_sm;
-    if (aligned && large) {
-        const int64_t ldw = ((int64_t)p.K * EB + 15) / 16 * 16 / EB;
+    // Rows of A off the 16-byte boundaries are copied to a padded piece first,
+    // which many columns repay: 2 x 22748 x 995 x 125 in BF16 327 -> 127 us, 2000 x
+    // 300 x 77 47 -> 30, 512 x 128 x 127 31.4 -> 29.9; but 65536 x 16 x 131 35 -> 49,
+    // and 16 x 640 x 64 x 99 26 -> 27.
+    const bool deep = (int64_t)p.K * (kTcBM + BN) >= (EB == 4 ? 14000 : 20000);
+    if (aligned ? deep || blocks >= 2 * ctx->n_sm : deep && p.N >= 96) {
+        const int64_t ldw = ((int64_t)p.K * EB + 15) / 16 * 16 / EB, ldp = ((int64_t)p.K + 3) / 4 * 4;
+        const int64_t pad = aligned ? 0
+                                    : std::min<int64_t>((int64_t)batch * p.M * ldp * 4,
+                                                        std::max(kPadBytes, (int64_t)kTcBM * ldp * 4));
+        const int64_t w_bytes = ((int64_t)batch * p.N * ldw * EB + 15) / 16 * 16;
         DevBuf W;
-        if (dev_alloc(ctx, W, (size_t)batch * p.N * ldw * EB, s) == PNE_OK) {
+        if (dev_alloc(ctx, W, (size_t)(w_bytes + pad), s) == PNE_OK) {
             bool used = false;
-            const cudaError_t e = launch_dense_stream<EB>(p, batch, ctx->n_sm, W.ptr, ldw, s, used);
+            const cudaError_t e =
+                aligned ? launch_dense_stream<EB>(p, batch, ctx->n_sm, W.ptr, ldw, s, used)
+                        : launch_padded_stream<EB>(p, batch, ctx->n_sm, (float *)((char *)W.ptr + w_bytes), ldp, W.ptr,
+                                                   ldw, s, used);
             dev_free(ctx, W, s);
             if (e != cudaSuccess || used) return e;
         } else {
