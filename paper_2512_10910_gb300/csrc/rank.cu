@@ -62,7 +62,7 @@ constexpr int kWpLd = kWpDim + 1;       // column stride of the Jacobi matrices 
 struct WPShare {
     double R[kWpCluster][kWpDim * kWpDim];      // triangles of each block's rows, side A then side B
     double RB[kWpCluster][kWpDim * kWpDim];
-    double WB[kWpDim * kWpDim], sB[kWpDim];     // U_B S_B (column c at c * kWpDim) and S_B
+    double WB[kWpDim * kWpDim], sB[kWpDim];     // U_B (column c at c * kWpDim) and S_B
     double XL[kWpDim * kWpDim], XR[kWpDim * kWpDim];   // leg transforms [in][out]
     int code;                                   // 0 next bond, 1 a zero singular value, 2 converged
 };
@@ -226,8 +226,9 @@ __device__ void qr_rows(const Load &load, int rows, int d, QrShared &q)
 // two, so a round is as long as the FP64 instructions of one warp: the sums
 // halve their list at each exchange (5 additions for the three inner products,
 // not 12), and what only decides how fast the columns become orthogonal -- the
-// angle -- is FP32, taken from the bits of the FP64 sums; cosine and sine (c^2 +
-// s^2 = 1 to FP64's rounding) and the rotation are FP64.  At n = 16 a
+// angle -- starts in FP32, taken from the bits of the FP64 sums, with one FP64
+// correction; cosine and sine (c^2 + s^2 = 1 to FP64's rounding) and the rotation
+// are FP64.  At n = 16 a
 // round on one warp, four rows to a lane and all FP64, took 5.2 k clocks (two
 // thirds of a bond update: 1.03 M of 1.5 M clocks).
 struct JacobiPair {
@@ -264,9 +265,8 @@ __device__ __forceinline__ double widen(float x)        // normal x
 }
 
 // On return the columns of W are orthogonal, sorted by their norms (sig)
-// descending; with ACC the rotations are accumulated on V (identity on entry,
-// the same layout), whose columns move along.  The whole block.
-template <bool ACC>
+// descending; the rotations are accumulated on V (identity on entry, the same
+// layout), whose columns move along.  The whole block.
 __device__ void jacobi_columns(double *W, double *V, double *sig, int n)
 {
     const int lane = threadIdx.x & 31, pr = threadIdx.x >> 4, row = threadIdx.x & 15, base = lane & 16;
@@ -305,9 +305,15 @@ __device__ void jacobi_columns(double *W, double *V, double *sig, int n)
                 const float t = (hf < 0.f ? -g2 : g2) / (fabsf(hf) + sqrtf(fmaf(hf, hf, g2 * g2)));
                 double cs, sn;
                 if (fabsf(t) >= 1e-18f && fabsf(t) <= 1.5f) {
-                    // c = rsqrt(1 + t^2) and s = t c in FP32 miss c^2 + s^2 = 1 by r = O(1e-7), which
-                    // (1 + r)^(-1/2) to second order corrects; t c and c^2 are exact in FP64
-                    const double c = widen(rsqrtf(fmaf(t, t, 1.f))), s = widen(t) * c;
+                    // a Newton step on g t^2 + h t - g takes t from FP32 to FP64 (its residual in
+                    // FP64, its slope in FP32): a small entry of V is a few such t, and the leg
+                    // transforms divide it by a weight as small, so it has to be right to its own size
+                    const double t0 = widen(t), res = fma(fma(g, t0, h), t0, -g);
+                    const float dt = -scaled_float(res, eh) / fmaf(g2, t, hf);
+                    const double td = t0 + (fabsf(dt) >= 1e-36f ? widen(dt) : 0.0);
+                    // c = rsqrt(1 + t^2) in FP32 and s = t c miss c^2 + s^2 = 1 by r = O(1e-7), which
+                    // (1 + r)^(-1/2) to second order corrects
+                    const double c = widen(rsqrtf(fmaf(t, t, 1.f))), s = td * c;
                     const double r = fma(s, s, fma(c, c, -1.0));
                     const double k = fma(r, fma(r, 0.375, -0.5), 1.0);
                     cs = c * k;
@@ -319,7 +325,7 @@ __device__ void jacobi_columns(double *W, double *V, double *sig, int n)
                 if (row < n) {
                     *wp = cs * x - sn * y;
                     *wq = sn * x + cs * y;
-                    if (ACC) {
+                    {
                         double *vp = V + p.c0 * kWpLd + row, *vq = V + p.c1 * kWpLd + row;
                         const double vx = *vp, vy = *vq;
                         *vp = cs * vx - sn * vy;
@@ -349,14 +355,14 @@ __device__ void jacobi_columns(double *W, double *V, double *sig, int n)
     if (lane < n)
         for (int row = 0; row < n; ++row) {
             col[row] = W[lane * kWpLd + row];
-            if (ACC) vcol[row] = V[lane * kWpLd + row];
+            vcol[row] = V[lane * kWpLd + row];
         }
     __syncwarp();
     if (lane < n) {
         sig[at] = norm;
         for (int row = 0; row < n; ++row) {
             W[at * kWpLd + row] = col[row];
-            if (ACC) V[at * kWpLd + row] = vcol[row];
+            V[at * kWpLd + row] = vcol[row];
         }
     }
     __syncwarp();
@@ -461,8 +467,10 @@ __global__ void __launch_bounds__(kWpThreads) weight_passing_kernel(WPParams p, 
             if (split_a) share_rows(sa, sh.R);
             if (split_b) share_rows(sb, sh.RB);
             if (split_a || split_b) wp_barrier(blocks);
-            // the triangle of one side to V S, the columns of its transpose after the rotations
-            auto side = [&](const WPSite &s, bool split, const double (*R)[kWpDim * kWpDim], double *W, double *sig) {
+            // The right vectors V and singular values of one side's triangle.  V is the product of
+            // the rotations: its small entries are right to their own size, which the columns of
+            // R^T Q / S = V are not, and the leg transforms divide them by weights as small.
+            auto side = [&](const WPSite &s, bool split, const double (*R)[kWpDim * kWpDim], double *V, double *sig) {
                 if (split)
                     qr_rows<DM>([&](int row, double (&x)[DM]) {
 #pragma unroll
@@ -471,9 +479,12 @@ __global__ void __launch_bounds__(kWpThreads) weight_passing_kernel(WPParams p, 
                     }, blocks * d, d, q);
                 else
                     qr_rows<DM>(rows_of(s, 0), s.rest, d, q);
-                for (int e = tid; e < d * d; e += kWpThreads) W[e / d * kWpLd + e % d] = q.R[e / d][e % d];
+                for (int e = tid; e < d * d; e += kWpThreads) {
+                    WC[e % d * kWpLd + e / d] = q.R[e / d][e % d];
+                    V[e / d * kWpLd + e % d] = e / d == e % d ? 1.0 : 0.0;
+                }
                 __syncthreads();
-                jacobi_columns<false>(W, nullptr, sig, d);
+                jacobi_columns(WC, V, sig, d);
                 __syncthreads();
             };
             const int rank_b = blocks > 1 ? 1 : 0;
@@ -500,11 +511,11 @@ __global__ void __launch_bounds__(kWpThreads) weight_passing_kernel(WPParams p, 
                     const int a = e / d, c = e % d;
                     double acc = 0.0;
                     for (int x = 0; x < d; ++x) acc = fma(WA[a * kWpLd + x] * __ldcg(Si + x), WBs[c * kWpLd + x], acc);
-                    WC[c * kWpLd + a] = acc;
+                    WC[c * kWpLd + a] = sA[a] * acc * sB[c];
                     VC[c * kWpLd + a] = a == c ? 1.0 : 0.0;
                 }
                 __syncthreads();
-                if (!bad_sh) jacobi_columns<true>(WC, VC, sC, d);          // WC -> U_C S_C, VC = V_C
+                if (!bad_sh) jacobi_columns(WC, VC, sC, d);          // WC -> U_C S_C, VC = V_C
                 if (!bad_sh && tid < 32) {
                     const double s = tid < d ? sC[tid] : 0.0;
                     if (!(sC[d - 1] > 1e-300)) bad_sh = 1;
@@ -525,8 +536,8 @@ __global__ void __launch_bounds__(kWpThreads) weight_passing_kernel(WPParams p, 
                     // right = S_C^{(1-alpha)/2} V_C^T S_B^{-1} U_B^T on B's, as [in][out]
                     for (int e = tid; e < d * d; e += kWpThreads) {
                         const int c = e / d, at = c * kWpLd + e % d;
-                        WA[at] = WA[at] / sA[c] / sA[c];
-                        WBs[at] = WBs[at] / sB[c] / sB[c];
+                        WA[at] = WA[at] / sA[c];
+                        WBs[at] = WBs[at] / sB[c];
                         WC[at] = WC[at] / sC[c];
                     }
                     __syncthreads();
