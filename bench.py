@@ -676,7 +676,7 @@ def run_rank_r_extra(args, ctx, pne, torch, dev, local_rank):
     wp_ms = a.elapsed_time(b)
     _, sw, _ = pne.pne_weights_read(ctx.h, w, len(nets), int(g.n_bonds))
     out["weight_passing"] = {"ms_per_step": wp_ms, "max_sweeps": int(np.max(sw)),
-                             "how": "one block per tensor set, bonds in id order (FP64 QR and Jacobi SVDs)"}
+                             "how": "a cluster of blocks per tensor set, bonds in id order (FP64 QR and Jacobi SVDs)"}
     try:
         for form, parts, name in ((0, I.square3x3_pinwheel(), "linear_4_single_index"),
                                   (1, I.square3x3_six_lines(), "combinatorial_6_multi_index")):
