@@ -28,6 +28,7 @@
 #include <string>
 #include <vector>
 
+#include "jacobi.h"
 #include "pne_internal.h"
 
 struct pne_weights {
@@ -225,12 +226,9 @@ __device__ void qr_rows(const Load &load, int rows, int d, QrShared &q)
 // 64 clocks on this GPU (two lanes per clock and SM), an FP32 or integer one
 // two, so a round is as long as the FP64 instructions of one warp: the sums
 // halve their list at each exchange (5 additions for the three inner products,
-// not 12), and what only decides how fast the columns become orthogonal -- the
-// angle -- starts in FP32, taken from the bits of the FP64 sums, with one FP64
-// correction; cosine and sine (c^2 + s^2 = 1 to FP64's rounding) and the rotation
-// are FP64.  At n = 16 a
-// round on one warp, four rows to a lane and all FP64, took 5.2 k clocks (two
-// thirds of a bond update: 1.03 M of 1.5 M clocks).
+// not 12), and the rotation takes ten (jacobi_rotation).  At n = 16 a round on
+// one warp, four rows to a lane, took 5.2 k clocks (two thirds of a bond update:
+// 1.03 M of 1.5 M clocks).
 struct JacobiPair {
     int c0, c1;
     bool on;
@@ -246,22 +244,6 @@ __device__ __forceinline__ JacobiPair jacobi_pair(int pr, int rd, int n, int n2)
     c1 = pr == 0 ? rd : (c1 >= m ? c1 - m : c1);
     const int lo = c0 < c1 ? c0 : c1, hi = c0 < c1 ? c1 : c0;
     return {lo, hi, pr < n2 / 2 && hi < n};
-}
-
-__device__ __forceinline__ int double_exponent(double x) { return (__double2hiint(x) >> 20) & 0x7ff; }
-
-// x 2^(1023 - e) truncated to FP32 (0 below FP32's range), and back, by bits
-__device__ __forceinline__ float scaled_float(double x, int e)
-{
-    const int hi = __double2hiint(x), ex = ((hi >> 20) & 0x7ff) - e + 127;
-    if (ex <= 0) return 0.f;
-    return __int_as_float((hi & 0x80000000) | (min(ex, 254) << 23) | ((hi & 0xfffff) << 3) |
-                          (int)((unsigned)__double2loint(x) >> 29));
-}
-__device__ __forceinline__ double widen(float x)        // normal x
-{
-    const int b = __float_as_int(x);
-    return __hiloint2double((b & 0x80000000) | ((((b >> 23) & 0xff) + 896) << 20) | ((b & 0x7fffff) >> 3), b << 29);
 }
 
 // On return the columns of W are orthogonal, sorted by their norms (sig)
@@ -298,30 +280,8 @@ __device__ void jacobi_columns(double *W, double *V, double *sig, int n)
             if (af == 0.f || bf == 0.f) small = fabs(g) <= 1e-15 * sqrt(a) * sqrt(b);   // norms 2^63 apart
             const bool turn = p.on && !(small || g == 0.0);
             if (turn) {
-                // tangent of the rotation that takes g to zero: t = sign(z) / (|z| + sqrt(1 + z^2)), z = h / (2 g)
-                const double h = b - a;
-                const int eh = max(double_exponent(h), double_exponent(g));
-                const float hf = scaled_float(h, eh), g2 = 2.f * scaled_float(g, eh);
-                const float t = (hf < 0.f ? -g2 : g2) / (fabsf(hf) + sqrtf(fmaf(hf, hf, g2 * g2)));
                 double cs, sn;
-                if (fabsf(t) >= 1e-18f && fabsf(t) <= 1.5f) {
-                    // a Newton step on g t^2 + h t - g takes t from FP32 to FP64 (its residual in
-                    // FP64, its slope in FP32): a small entry of V is a few such t, and the leg
-                    // transforms divide it by a weight as small, so it has to be right to its own size
-                    const double t0 = widen(t), res = fma(fma(g, t0, h), t0, -g);
-                    const float dt = -scaled_float(res, eh) / fmaf(g2, t, hf);
-                    const double td = t0 + (fabsf(dt) >= 1e-36f ? widen(dt) : 0.0);
-                    // c = rsqrt(1 + t^2) in FP32 and s = t c miss c^2 + s^2 = 1 by r = O(1e-7), which
-                    // (1 + r)^(-1/2) to second order corrects
-                    const double c = widen(rsqrtf(fmaf(t, t, 1.f))), s = td * c;
-                    const double r = fma(s, s, fma(c, c, -1.0));
-                    const double k = fma(r, fma(r, 0.375, -0.5), 1.0);
-                    cs = c * k;
-                    sn = s * k;
-                } else {                                 // graded beyond FP32: t = g / h to rounding
-                    cs = 1.0;
-                    sn = g / h;
-                }
+                jacobi_rotation(a, b, g, cs, sn);
                 if (row < n) {
                     *wp = cs * x - sn * y;
                     *wq = sn * x + cs * y;
