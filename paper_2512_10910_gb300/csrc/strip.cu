@@ -35,6 +35,7 @@
 #include <string>
 #include <vector>
 
+#include "float_float.h"
 #include "pne_internal.h"
 
 namespace pne {
@@ -240,28 +241,15 @@ struct ApplyParams {
 
 // out[p][o][s] = sum_i mat[o][i] * in[p][i][s] (* scale): one site of the row.
 // IN / OUT formats: 0 FP64, 1 float-float pair (hi, lo) in the same 8 bytes.
-// With FF the multiply-adds run on the FP32 pipes as compensated dot products:
-// the running sum by Knuth's two-sum, whose second difference is taken from
-// the unrounded product by an FMA and so carries the product's own rounding
-// too, the error terms and the low-part cross products gathered in one FP32
-// compensation: about 2^-48 relative to sum |a x| per output, where the FP64
-// pipe of this part retires 1/60 of the FP32 rate.  That is ten instructions a
-// multiply-add; with the product split by an FMA of its own it was twelve, and
-// no more exact.  The FP32 pipes bound it (63% busy, 72% of the issue slots: the
-// rest is lost to operand conflicts), so the matrix comes in 16-byte loads of
-// two entries' pairs and an index costs one 32-bit division.  Row products of a
-// call, ms before and now: chi 4, 7 wide, 8 tensors 7.2, 5.6; 10 wide 86, 77;
-// chi 5, 8 wide, 2 tensors 17.8, 13.5; chi 8, 6 wide, 2 tensors 26.2, 17.6.
-// Packed FP32 instructions (two fibres a thread) were slower, 82 ms at chi 4,
-// 10 wide, and so was taking few enough tensors at a time to stay in L2 (88).
-struct ffp { float h, l; };
-
-__device__ __forceinline__ ffp split_double(double x)
-{
-    const float h = __double2float_rn(x);
-    return {h, __double2float_rn(x - (double)h)};
-}
-
+// With FF the multiply-adds are float-float (ff_dot).  The FP32 pipes bound it at
+// chi >= 4 (63% busy, 72% of the issue slots: the rest is lost to operand conflicts), so
+// the matrix comes in 16-byte loads of two entries' pairs and an index costs one 32-bit
+// division.  Row products of a call, ms, with 8-byte loads, 64-bit divisions, blocks of
+// 256 threads and twelve instructions a multiply-add everywhere, and now: chi 4, 7 wide,
+// 8 tensors 7.2, 5.6; 10 wide 86, 77; chi 5, 8 wide, 2 tensors 17.8, 13.4; chi 8, 6
+// wide, 2 tensors 26.2, 17.6.  Packed FP32 instructions (two fibres a thread) were
+// slower, 82 ms at chi 4, 10 wide, and so was taking few enough tensors at a time to
+// stay in L2 (88).
 template <int NIN, int NOUT, int IN_FF, int OUT_FF>
 __global__ void __launch_bounds__(kApplyThreads) strip_apply_kernel(ApplyParams p)
 {
@@ -320,33 +308,19 @@ __global__ void __launch_bounds__(kApplyThreads) strip_apply_kernel(ApplyParams 
             }
 #pragma unroll 2
             for (int o = 0; o < NOUT; ++o) {
-                float sh = 0.f, c = 0.f;
+                ff_dot<NIN> dot;
 #pragma unroll
                 for (int i = 0; i < NIN; ++i) {
                     const float4 m = Mf[o * kPairs + i / 2];
-                    const float ah = i & 1 ? m.z : m.x, al = i & 1 ? m.w : m.y;
-                    const float pr = __fmul_rn(ah, xh[i]);
-                    if (i == 0) {
-                        sh = pr;
-                        c = __fmaf_rn(ah, xh[i], -pr);
-                    } else {
-                        const float t = __fadd_rn(sh, pr);
-                        const float bb = __fsub_rn(t, sh);
-                        const float e = __fmaf_rn(ah, xh[i], -bb);   // the product's share of t's error, and its own
-                        c = __fadd_rn(c, __fadd_rn(__fsub_rn(sh, __fsub_rn(t, bb)), e));
-                        sh = t;
-                    }
-                    c = __fmaf_rn(ah, xl[i], c);
-                    c = __fmaf_rn(al, xh[i], c);
+                    dot.term(i, i & 1 ? m.z : m.x, i & 1 ? m.w : m.y, xh[i], xl[i]);
                 }
-                const float hi = __fadd_rn(sh, c);
-                const float lo = __fsub_rn(c, __fsub_rn(hi, sh));
+                const ffp v = dot.value();
                 if (OUT_FF) {
                     float2 *out = reinterpret_cast<float2 *>(p.out + b * p.out_stride) + dst0;
-                    out[o * p.S] = make_float2(hi, lo);
+                    out[o * p.S] = make_float2(v.h, v.l);
                 } else {
                     double *out = p.out + b * p.out_stride + dst0;
-                    out[o * p.S] = (double)hi + (double)lo;
+                    out[o * p.S] = (double)v.h + (double)v.l;
                 }
             }
         }
