@@ -425,7 +425,8 @@ void pne_server_destroy(pne_server *s);
  *          tensor sets; every bond dimension at most 16 and at most the
  *          product of the other dimensions of either of its tensors.
  *   alpha  in (0, 1] (the paper's benchmarks use 0.8); tol > 0; max_sweeps > 0.
- * FP64 throughout.  Synchronises `stream`.  Returns PNE_ENOCONV (handle
+ * FP64 throughout; a set's weights, sweeps and scale do not depend on the
+ * other sets of its batch.  Synchronises `stream`.  Returns PNE_ENOCONV (handle
  * still returned) when some set did not reach tol, PNE_EDEGENERATE when a
  * tensor is rank-deficient across a bond (a zero singular value). */
 typedef struct pne_weights pne_weights;
