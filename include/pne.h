@@ -428,7 +428,8 @@ void pne_server_destroy(pne_server *s);
  * FP64 throughout; a set's weights, sweeps and scale do not depend on the
  * other sets of its batch.  Synchronises `stream`.  Returns PNE_ENOCONV (handle
  * still returned) when some set did not reach tol, PNE_EDEGENERATE when a
- * tensor is rank-deficient across a bond (a zero singular value). */
+ * tensor is rank-deficient across a bond (a zero singular value) or a singular
+ * value's square overflows. */
 typedef struct pne_weights pne_weights;
 pne_status pne_weight_passing(pne_ctx *ctx, const pne_network *net, double alpha, double tol, int32_t max_sweeps,
                               void *stream, pne_weights **out);

@@ -1,9 +1,15 @@
-// The rotation of a one-sided Jacobi step, in few FP64 instructions.
+// One-sided Jacobi of small matrices, in few FP64 instructions.
 #pragma once
 
 #include <cuda_runtime.h>
 
+#include <cmath>
+
 namespace pne {
+
+constexpr int kJacobiDim = 16;               // most columns and rows
+constexpr int kJacobiThreads = 128;          // of the block
+constexpr int kJacobiLd = kJacobiDim + 1;    // column stride in shared memory
 
 __device__ __forceinline__ int double_exponent(double x) { return (__double2hiint(x) >> 20) & 0x7ff; }
 
@@ -57,6 +63,117 @@ __device__ __forceinline__ void jacobi_rotation(double a, double b, double g, do
         cs = 1.0;
         sn = g / h;
     }
+}
+
+// ---- one-sided Jacobi (Hestenes) of the columns of a matrix in shared memory
+// (entry (row, c) at c * kJacobiLd + row).  A round of the tournament rotates up to
+// eight disjoint pairs at once, sixteen threads to a pair and a row each: the
+// four warps of the block.  An FP64 instruction takes a warp's scheduler about
+// 64 clocks on this GPU (two lanes per clock and SM), an FP32 or integer one
+// two, so a round is as long as the FP64 instructions of one warp: the sums
+// halve their list at each exchange (5 additions for the three inner products,
+// not 12), and the rotation takes ten (jacobi_rotation).  At n = 16 a round on
+// one warp, four rows to a lane, took 5.2 k clocks (two thirds of a bond update:
+// 1.03 M of 1.5 M clocks).
+struct JacobiPair {
+    int c0, c1;
+    bool on;
+};
+
+// Pair `pr` of round rd among n columns (n2 = n rounded up to even): the circle
+// method; an odd n leaves one column out.
+__device__ __forceinline__ JacobiPair jacobi_pair(int pr, int rd, int n, int n2)
+{
+    const int m = n2 - 1;
+    int c0 = rd + pr, c1 = rd + m - pr;
+    c0 = pr == 0 ? m : (c0 >= m ? c0 - m : c0);
+    c1 = pr == 0 ? rd : (c1 >= m ? c1 - m : c1);
+    const int lo = c0 < c1 ? c0 : c1, hi = c0 < c1 ? c1 : c0;
+    return {lo, hi, pr < n2 / 2 && hi < n};
+}
+
+// On return the columns of W are orthogonal, sorted by their norms (sig)
+// descending; the rotations are accumulated on V (identity on entry, the same
+// layout), whose columns move along.  The whole block.
+__device__ inline void jacobi_columns(double *W, double *V, double *sig, int n)
+{
+    const int lane = threadIdx.x & 31, pr = threadIdx.x >> 4, row = threadIdx.x & 15, base = lane & 16;
+    const int n2 = n + (n & 1), rounds = n2 - 1;
+    for (int sweep = 0; sweep < 60 && n > 1; ++sweep) {
+        int rotated = 0;
+        for (int rd = 0; rd < rounds; ++rd) {
+            const JacobiPair p = jacobi_pair(pr, rd, n, n2);
+            const bool in = p.on && row < n;
+            double *wp = W + p.c0 * kJacobiLd + row, *wq = W + p.c1 * kJacobiLd + row;
+            const double x = in ? *wp : 0.0, y = in ? *wq : 0.0;
+            // sums over the 16 rows of x^2, y^2 and x y
+            double s0 = x * x, s1 = y * y;
+            const double s2 = x * y;
+            const bool u8 = lane & 8, u4 = lane & 4;
+            double g0 = __shfl_xor_sync(0xffffffffu, u8 ? s0 : s2, 8), g1 = __shfl_xor_sync(0xffffffffu, s1, 8);
+            s0 = (u8 ? s2 : s0) + g0;
+            s1 = s1 + g1;
+            g0 = __shfl_xor_sync(0xffffffffu, u4 ? s0 : s1, 4);
+            s0 = (u4 ? s1 : s0) + g0;                 // lanes 0: x^2, 4: y^2, 8: x y
+            s0 += __shfl_xor_sync(0xffffffffu, s0, 2);
+            s0 += __shfl_xor_sync(0xffffffffu, s0, 1);
+            const double a = __shfl_sync(0xffffffffu, s0, base), b = __shfl_sync(0xffffffffu, s0, base + 4),
+                         g = __shfl_sync(0xffffffffu, s0, base + 8);
+            // |g| <= 1e-15 sqrt(a b)
+            const int e = max(double_exponent(a), double_exponent(b));
+            const float af = scaled_float(a, e), bf = scaled_float(b, e), gf = scaled_float(g, e);
+            bool small = fabsf(gf) <= 1e-15f * sqrtf(af) * sqrtf(bf);
+            if (af == 0.f || bf == 0.f) small = fabs(g) <= 1e-15 * sqrt(a) * sqrt(b);   // norms 2^63 apart
+            const bool turn = p.on && !(small || g == 0.0);
+            if (turn) {
+                double cs, sn;
+                jacobi_rotation(a, b, g, cs, sn);
+                if (row < n) {
+                    *wp = cs * x - sn * y;
+                    *wq = sn * x + cs * y;
+                    {
+                        double *vp = V + p.c0 * kJacobiLd + row, *vq = V + p.c1 * kJacobiLd + row;
+                        const double vx = *vp, vy = *vq;
+                        *vp = cs * vx - sn * vy;
+                        *vq = sn * vx + cs * vy;
+                    }
+                }
+            }
+            rotated |= __syncthreads_or(turn);
+        }
+        if (!rotated) break;
+    }
+    if (threadIdx.x >= 32) return;
+    __syncwarp();
+    // norms, a column per lane, and the descending order (ties by index; a NaN
+    // counts as infinite, so that every place is filled)
+    double norm = -1.0;
+    if (lane < n) {
+        double s2 = 0.0;
+        for (int row = 0; row < n; ++row) s2 = fma(W[lane * kJacobiLd + row], W[lane * kJacobiLd + row], s2);
+        norm = sqrt(s2);
+    }
+    const double key = norm == norm ? norm : INFINITY;
+    int at = 0;
+    for (int c = 0; c < n; ++c) {
+        const double o = __shfl_sync(0xffffffffu, key, c);
+        at += (o > key || (o == key && c < lane)) ? 1 : 0;
+    }
+    double col[kJacobiDim], vcol[kJacobiDim];
+    if (lane < n)
+        for (int row = 0; row < n; ++row) {
+            col[row] = W[lane * kJacobiLd + row];
+            vcol[row] = V[lane * kJacobiLd + row];
+        }
+    __syncwarp();
+    if (lane < n) {
+        sig[at] = norm;
+        for (int row = 0; row < n; ++row) {
+            W[at * kJacobiLd + row] = col[row];
+            V[at * kJacobiLd + row] = vcol[row];
+        }
+    }
+    __syncwarp();
 }
 
 }  // namespace pne

@@ -50,14 +50,14 @@ pne_status geometry_for(pne_ctx *ctx, const pne_network *net, cudaStream_t s, st
 
 namespace {
 
-constexpr int kWpDim = 16;              // largest bond dimension of weight passing
-constexpr int kWpThreads = 128;
+constexpr int kWpDim = kJacobiDim;      // largest bond dimension of weight passing
+constexpr int kWpThreads = kJacobiThreads;
 constexpr int kWpWarps = kWpThreads / 32;
 constexpr int kWpRows = 4;              // rows a thread holds during the QR
 constexpr int kWpPanel = kWpThreads * kWpRows;
 constexpr int kWpCluster = 8;           // most blocks per tensor set (portable cluster size)
 constexpr int kWpParts = kWpCluster;    // most parts of a matrix's rows
-constexpr int kWpLd = kWpDim + 1;       // column stride of the Jacobi matrices in shared memory
+constexpr int kWpLd = kJacobiLd;
 
 // What the blocks of one set pass to each other, in global memory (read past
 // L1), each field written between two cluster barriers and read after them.
@@ -66,7 +66,7 @@ struct WPShare {
     double RB[kWpParts][kWpDim * kWpDim];
     double WB[kWpDim * kWpDim], sB[kWpDim];     // U_B (column c at c * kWpDim) and S_B
     double XL[kWpDim * kWpDim], XR[kWpDim * kWpDim];   // leg transforms [in][out]
-    int code;                                   // 0 next bond, 1 a zero singular value, 2 converged
+    int code;                                   // 0 next bond, 1 a bad singular value, 2 converged
 };
 
 struct WPParams {
@@ -81,7 +81,7 @@ struct WPParams {
     int max_sweeps;
     double *log_scale;         // [n_sets]
     int32_t *sweeps;           // [n_sets] (0: not converged)
-    int32_t *flags;            // [n_sets] 1: a zero singular value
+    int32_t *flags;            // [n_sets] 1: a zero singular value, or one that is not finite
 };
 
 __device__ __forceinline__ void wp_barrier(int blocks)
@@ -218,115 +218,6 @@ __device__ void qr_rows(const Load &load, int rows, int d, QrShared &q)
         qr_columns<DM, 0>(x, nr, q, d);
     }
     __syncthreads();
-}
-
-// ---- one-sided Jacobi (Hestenes) of the columns of a matrix in shared memory
-// (entry (row, c) at c * kWpLd + row).  A round of the tournament rotates up to
-// eight disjoint pairs at once, sixteen threads to a pair and a row each: the
-// four warps of the block.  An FP64 instruction takes a warp's scheduler about
-// 64 clocks on this GPU (two lanes per clock and SM), an FP32 or integer one
-// two, so a round is as long as the FP64 instructions of one warp: the sums
-// halve their list at each exchange (5 additions for the three inner products,
-// not 12), and the rotation takes ten (jacobi_rotation).  At n = 16 a round on
-// one warp, four rows to a lane, took 5.2 k clocks (two thirds of a bond update:
-// 1.03 M of 1.5 M clocks).
-struct JacobiPair {
-    int c0, c1;
-    bool on;
-};
-
-// Pair `pr` of round rd among n columns (n2 = n rounded up to even): the circle
-// method; an odd n leaves one column out.
-__device__ __forceinline__ JacobiPair jacobi_pair(int pr, int rd, int n, int n2)
-{
-    const int m = n2 - 1;
-    int c0 = rd + pr, c1 = rd + m - pr;
-    c0 = pr == 0 ? m : (c0 >= m ? c0 - m : c0);
-    c1 = pr == 0 ? rd : (c1 >= m ? c1 - m : c1);
-    const int lo = c0 < c1 ? c0 : c1, hi = c0 < c1 ? c1 : c0;
-    return {lo, hi, pr < n2 / 2 && hi < n};
-}
-
-// On return the columns of W are orthogonal, sorted by their norms (sig)
-// descending; the rotations are accumulated on V (identity on entry, the same
-// layout), whose columns move along.  The whole block.
-__device__ void jacobi_columns(double *W, double *V, double *sig, int n)
-{
-    const int lane = threadIdx.x & 31, pr = threadIdx.x >> 4, row = threadIdx.x & 15, base = lane & 16;
-    const int n2 = n + (n & 1), rounds = n2 - 1;
-    for (int sweep = 0; sweep < 60 && n > 1; ++sweep) {
-        int rotated = 0;
-        for (int rd = 0; rd < rounds; ++rd) {
-            const JacobiPair p = jacobi_pair(pr, rd, n, n2);
-            const bool in = p.on && row < n;
-            double *wp = W + p.c0 * kWpLd + row, *wq = W + p.c1 * kWpLd + row;
-            const double x = in ? *wp : 0.0, y = in ? *wq : 0.0;
-            // sums over the 16 rows of x^2, y^2 and x y
-            double s0 = x * x, s1 = y * y;
-            const double s2 = x * y;
-            const bool u8 = lane & 8, u4 = lane & 4;
-            double g0 = __shfl_xor_sync(0xffffffffu, u8 ? s0 : s2, 8), g1 = __shfl_xor_sync(0xffffffffu, s1, 8);
-            s0 = (u8 ? s2 : s0) + g0;
-            s1 = s1 + g1;
-            g0 = __shfl_xor_sync(0xffffffffu, u4 ? s0 : s1, 4);
-            s0 = (u4 ? s1 : s0) + g0;                 // lanes 0: x^2, 4: y^2, 8: x y
-            s0 += __shfl_xor_sync(0xffffffffu, s0, 2);
-            s0 += __shfl_xor_sync(0xffffffffu, s0, 1);
-            const double a = __shfl_sync(0xffffffffu, s0, base), b = __shfl_sync(0xffffffffu, s0, base + 4),
-                         g = __shfl_sync(0xffffffffu, s0, base + 8);
-            // |g| <= 1e-15 sqrt(a b)
-            const int e = max(double_exponent(a), double_exponent(b));
-            const float af = scaled_float(a, e), bf = scaled_float(b, e), gf = scaled_float(g, e);
-            bool small = fabsf(gf) <= 1e-15f * sqrtf(af) * sqrtf(bf);
-            if (af == 0.f || bf == 0.f) small = fabs(g) <= 1e-15 * sqrt(a) * sqrt(b);   // norms 2^63 apart
-            const bool turn = p.on && !(small || g == 0.0);
-            if (turn) {
-                double cs, sn;
-                jacobi_rotation(a, b, g, cs, sn);
-                if (row < n) {
-                    *wp = cs * x - sn * y;
-                    *wq = sn * x + cs * y;
-                    {
-                        double *vp = V + p.c0 * kWpLd + row, *vq = V + p.c1 * kWpLd + row;
-                        const double vx = *vp, vy = *vq;
-                        *vp = cs * vx - sn * vy;
-                        *vq = sn * vx + cs * vy;
-                    }
-                }
-            }
-            rotated |= __syncthreads_or(turn);
-        }
-        if (!rotated) break;
-    }
-    if (threadIdx.x >= 32) return;
-    __syncwarp();
-    // norms, a column per lane, and the descending order (ties by index)
-    double norm = -1.0;
-    if (lane < n) {
-        double s2 = 0.0;
-        for (int row = 0; row < n; ++row) s2 = fma(W[lane * kWpLd + row], W[lane * kWpLd + row], s2);
-        norm = sqrt(s2);
-    }
-    int at = 0;
-    for (int c = 0; c < n; ++c) {
-        const double o = __shfl_sync(0xffffffffu, norm, c);
-        at += (o > norm || (o == norm && c < lane)) ? 1 : 0;
-    }
-    double col[kWpDim], vcol[kWpDim];
-    if (lane < n)
-        for (int row = 0; row < n; ++row) {
-            col[row] = W[lane * kWpLd + row];
-            vcol[row] = V[lane * kWpLd + row];
-        }
-    __syncwarp();
-    if (lane < n) {
-        sig[at] = norm;
-        for (int row = 0; row < n; ++row) {
-            W[at * kWpLd + row] = col[row];
-            V[at * kWpLd + row] = vcol[row];
-        }
-    }
-    __syncwarp();
 }
 
 // A site's legs as one bond update needs them
@@ -473,9 +364,8 @@ __global__ void __launch_bounds__(kWpThreads) weight_passing_kernel(WPParams p, 
                     for (int e = tid; e < d * d; e += kWpThreads) WBs[e / d * kWpLd + e % d] = __ldcg(&sh.WB[e / d * kWpDim + e % d]);
                     if (tid < d) sB[tid] = __ldcg(&sh.sB[tid]);
                 }
-                if (tid == 0) bad_sh = 0;
                 __syncthreads();
-                if (tid < d && (!(sA[tid] > 1e-300) || !(sB[tid] > 1e-300))) bad_sh = 1;
+                const bool bad_side = tid < d && (!(sA[tid] > 1e-300) || !(sB[tid] > 1e-300));
                 // core M = S_A V_A^T S_i U_B S_B and its SVD
                 double *Si = Sset + (int64_t)b * kWpDim;
                 for (int e = tid; e < d * d; e += kWpThreads) {
@@ -485,24 +375,27 @@ __global__ void __launch_bounds__(kWpThreads) weight_passing_kernel(WPParams p, 
                     WC[c * kWpLd + a] = sA[a] * acc * sB[c];
                     VC[c * kWpLd + a] = a == c ? 1.0 : 0.0;
                 }
-                __syncthreads();
-                if (!bad_sh) jacobi_columns(WC, VC, sC, d);          // WC -> U_C S_C, VC = V_C
-                if (!bad_sh && tid < 32) {
+                const bool sides_ok = !__syncthreads_or(bad_side);
+                if (sides_ok) jacobi_columns(WC, VC, sC, d);         // WC -> U_C S_C, VC = V_C
+                if (sides_ok && tid < 32) {
                     const double s = tid < d ? sC[tid] : 0.0;
-                    if (!(sC[d - 1] > 1e-300)) bad_sh = 1;
                     const double w = tid < d ? pow(s, p.alpha) : 0.0;
                     if (tid < d) gC[tid] = pow(s, 0.5 * (1.0 - p.alpha));
                     double mx = w;
                     for (int off = 16; off > 0; off >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, off));
                     scale += log(mx);
                     const double nw = w / mx;
+                    // a zero singular value, or one that overflowed (fmax passes a NaN over)
+                    const bool bad = __any_sync(0xffffffffu, tid < d && (!(s > 1e-300) || nw != nw));
+                    if (tid == 0) bad_sh = bad;
                     double ch = tid < d ? fabs(nw - __ldcg(Si + tid)) : 0.0;
                     for (int off = 16; off > 0; off >>= 1) ch = fmax(ch, __shfl_xor_sync(0xffffffffu, ch, off));
                     change = fmax(change, ch);
                     if (tid < d) __stcg(Si + tid, nw);
                 }
                 __syncthreads();
-                if (!bad_sh) {
+                const bool ok = sides_ok && !bad_sh;
+                if (ok) {
                     // left = V_A S_A^{-1} U_C S_C^{(1-alpha)/2} on A's leg,
                     // right = S_C^{(1-alpha)/2} V_C^T S_B^{-1} U_B^T on B's, as [in][out]
                     for (int e = tid; e < d * d; e += kWpThreads) {
@@ -520,7 +413,7 @@ __global__ void __launch_bounds__(kWpThreads) weight_passing_kernel(WPParams p, 
                         __stcg((side_b ? sh.XR : sh.XL) + a * kWpDim + c, acc * gC[c]);
                     }
                 }
-                if (tid == 0) __stcg(&sh.code, bad_sh ? 1 : (b == p.n_bonds - 1 && change < p.tol ? 2 : 0));
+                if (tid == 0) __stcg(&sh.code, !ok ? 1 : (b == p.n_bonds - 1 && change < p.tol ? 2 : 0));
             }
             wp_barrier(blocks);
             code = __ldcg(&sh.code);
@@ -1065,7 +958,7 @@ pne_status pne_weight_passing(pne_ctx *ctx, const pne_network *net, double alpha
     w->last_stream = s;
     *out = w;
     for (int b = 0; b < B; ++b)
-        if (sw[B + b]) { set_error(ctx, PNE_EDEGENERATE, "a zero singular value in weight passing"); return PNE_EDEGENERATE; }
+        if (sw[B + b]) { set_error(ctx, PNE_EDEGENERATE, "a singular value in weight passing is zero or not finite"); return PNE_EDEGENERATE; }
     for (int b = 0; b < B; ++b)
         if (sw[b] == 0) { set_error(ctx, PNE_ENOCONV, "weight passing did not converge for a tensor set"); return PNE_ENOCONV; }
     return PNE_OK;
