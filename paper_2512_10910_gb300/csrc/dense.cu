@@ -1339,17 +1339,6 @@ cudaError_t launch_tc(pne_ctx *ctx, const GemmParams<float> &p, int batch, cudaS
     return cudaGetLastError();
 }
 
-// a word of pinned host memory per thread, or nullptr where none is to be had
-int *host_flag()
-{
-    thread_local int *word = nullptr;
-    if (!word && cudaHostAlloc((void **)&word, sizeof(int), cudaHostAllocPortable | cudaHostAllocMapped) != cudaSuccess) {
-        (void)cudaGetLastError();
-        word = nullptr;
-    }
-    return word;
-}
-
 template <int G, bool RING>
 cudaError_t launch_f64_units(const F64Params &p, dim3 grid, cudaStream_t s)
 {
@@ -1645,16 +1634,19 @@ pne_status pne_dense_gemm(pne_ctx *ctx, pne_dtype dtype, int32_t batch, int32_t 
     if (lda < K || ldb < K || ldc < N) return bad("leading dimensions below K (A, B) or N (C)");
     if (dtype == PNE_F32) return bad("dense_gemm takes PNE_F64, PNE_TF32 or PNE_BF16");
     cudaStream_t s = (cudaStream_t)stream;
-    // A wait that gave up is told in host memory where the kernel can write it:
-    // a word on the device takes a clear before and a copy after the product
-    // (BF16: 4 x 32768 x 256 x 256 73.6 us a call with them, 67 without;
-    // 128 x 16 x 16 31 and 17).
-    int *flag = host_flag();
+    // A wait of the tensor-core kernels that gave up is told in host memory where
+    // the kernel can write it: a word on the device takes a clear before and a copy
+    // after the product (BF16: 4 x 32768 x 256 x 256 80 us a call with them, 73 to
+    // 77 without; 128 x 16 x 16 31 and 17).  The word is the call's own, from the
+    // context's pool.
+    size_t flag_bytes = 0;
+    int *flag = dtype == PNE_F64 ? nullptr : (int *)take_pinned(ctx, sizeof(int), &flag_bytes);
     DevBuf err;
     cudaError_t e = cudaSuccess;
     if (flag) {
         *(volatile int *)flag = 0;
-    } else {
+    } else if (dtype != PNE_F64) {
+        (void)cudaGetLastError();
         const pne_status st = dev_alloc(ctx, err, 16, s);
         if (st) return st;
         e = cudaMemsetAsync(err.ptr, 0, 16, s);
@@ -1683,11 +1675,12 @@ pne_status pne_dense_gemm(pne_ctx *ctx, pne_dtype dtype, int32_t batch, int32_t 
         }
     }
     int herr = 0;
-    if (e == cudaSuccess && !flag) e = cudaMemcpyAsync(&herr, err.ptr, 4, cudaMemcpyDeviceToHost, s);
+    if (e == cudaSuccess && err.ptr) e = cudaMemcpyAsync(&herr, err.ptr, 4, cudaMemcpyDeviceToHost, s);
     const cudaError_t done = cudaStreamSynchronize(s);       // no kernel may write the word after the call
     if (e == cudaSuccess) e = done;
     if (flag) herr = *(volatile int *)flag;
-    else dev_free(ctx, err, s);
+    give_pinned(ctx, flag, flag_bytes);
+    dev_free(ctx, err, s);
     if (e != cudaSuccess) {
         set_error(ctx, PNE_ECUDA, std::string("dense_gemm: ") + cudaGetErrorString(e));
         return PNE_ECUDA;
