@@ -327,6 +327,18 @@ __global__ void close_starts_kernel(const int64_t *scanned, int64_t cap, const i
     starts[q] = q <= 2 ? 0 : (q <= K - 2 ? scanned[lv[q - 2]] : (q <= K ? scanned[(q - K + 2) * cap] : *total));
 }
 
+// The closing step's counts of the levels up to `level` (row 0: a node of level t
+// emits size t + 1) in the (size, node) table of the other forms, which is clear.
+__global__ void widen_counts_kernel(const int32_t *row0, const int64_t *lv, int level, int64_t cap, int32_t *counts)
+{
+    const int64_t n = lv[level];
+    for (int64_t u = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; u < n; u += (int64_t)gridDim.x * blockDim.x) {
+        int t = 1;
+        while (u >= lv[t]) ++t;                        // levels ascend with the arena position
+        counts[(t + 1) * cap + u] = row0[u];
+    }
+}
+
 // ---------------------------------------------------------------- search arena
 // Every prefix level lives in one node arena: level d (d = 1: the anchors,
 // one node per bond) is nodes[lv[d-1], lv[d]).  Level sizes stay on the
@@ -1342,10 +1354,9 @@ pne_status enumerate_clusters(pne_ctx *ctx, const Geometry &g, int K, int mode, 
     // prefix levels 1..D are expanded breadth-first; the last one closes the
     // three remaining sizes (LOOP mode, D == K - 3), only emits (D == K - 1) or
     // is searched depth-first (K - 1 > kPrefixMax)
-    bool fuse = mode == PNE_MODE_LOOP && K >= 4 && K - 3 <= kPrefixMax;
-    auto levels = [&] { return fuse ? K - 3 : ((K <= 1) ? 1 : std::min(kPrefixMax, K - 1)); };
-    int D = levels();
-    int final_kind = fuse ? 3 : ((K <= 1) ? 0 : (D == K - 1 ? 1 : 2));
+    const bool fuse = mode == PNE_MODE_LOOP && K >= 4 && K - 3 <= kPrefixMax;
+    const int D = fuse ? K - 3 : ((K <= 1) ? 1 : std::min(kPrefixMax, K - 1));
+    const int final_kind = fuse ? 3 : ((K <= 1) ? 0 : (D == K - 1 ? 1 : 2));
     const bool small = (K <= 12 && umax_need <= 64);
     // chunks of the blocked passes: one wave of resident blocks (the occupancy
     // is queried once per context)
@@ -1364,13 +1375,6 @@ pne_status enumerate_clusters(pne_ctx *ctx, const Geometry &g, int K, int mode, 
         auto it = ctx->arena_hint.find(hint_key);
         if (it != ctx->arena_hint.end()) cap = it->second;
     }
-    auto no_closing = [&] {           // the levels do not fit the largest arena: depth-first below one that does
-        fuse = false;
-        D = levels();
-        final_kind = D == K - 1 ? 1 : 2;
-        cap = INT64_MAX;
-    };
-    if (cap < 0) no_closing();        // known from the last search of this geometry
     const int64_t cap_max = ctx->arena_max > 0 ? std::max<int64_t>(ctx->arena_max, Mc) : kNodeCap;
     cap = std::min(cap_max, std::max<int64_t>(cap, Mc));
     Emit none{nullptr, nullptr, nullptr, rec.width, rec.vwidth};
@@ -1454,14 +1458,21 @@ pne_status enumerate_clusters(pne_ctx *ctx, const Geometry &g, int K, int mode, 
             dev_free(ctx, nodes, s); dev_free(ctx, tables, s); dev_free(ctx, counts, s); dev_free(ctx, base, s);
             continue;
         }
-        if (fuse) {
-            no_closing();
-            cap = cap_max;
-            dev_free(ctx, nodes, s); dev_free(ctx, tables, s); dev_free(ctx, counts, s); dev_free(ctx, base, s);
-            continue;
-        }
         // the largest arena holds levels 1..stop: search below level `stop` depth-first
         dfs_level = hb.ctl.stop;
+        if (fuse) {
+            DevBuf wide;
+            const size_t bytes = (size_t)(K + 1) * cap * 4;
+            if ((st = dev_alloc(ctx, wide, bytes, s))) return st;
+            const cudaError_t e = cudaMemsetAsync(wide.ptr, 0, bytes, s);
+            widen_counts_kernel<<<grid1(hb.lv[dfs_level], 256, ctx->n_sm), 256, 0, s>>>(A.counts, A.lv, dfs_level, cap,
+                                                                                       (int32_t *)wide.ptr);
+            dev_free(ctx, counts, s);
+            counts = wide;
+            A.counts = (int32_t *)wide.ptr;
+            PNE_CUDA_TRY(ctx, e);
+            PNE_LAUNCH_CHECK(ctx);
+        }
         dfs(A, dfs_level, 0, none);
         PNE_LAUNCH_CHECK(ctx);
         dev_free(ctx, base, s);
@@ -1473,8 +1484,7 @@ pne_status enumerate_clusters(pne_ctx *ctx, const Geometry &g, int K, int mode, 
         const int last = hb.ctl.stop ? hb.ctl.stop : D;
         const int64_t used = ((hb.lv[last] + 1023) / 1024) * 1024;
         std::lock_guard<std::mutex> lk(ctx->cache_mu);
-        const bool closing_failed = !fuse && mode == PNE_MODE_LOOP && K >= 4 && K - 3 <= kPrefixMax;
-        ctx->arena_hint[hint_key] = closing_failed ? -1 : hb.ctl.stop ? cap_max : std::max<int64_t>(used, 1024);
+        ctx->arena_hint[hint_key] = hb.ctl.stop ? cap_max : std::max<int64_t>(used, 1024);
     }
     uint64_t n_cl = 0;
     rec.size_start.assign(K + 2, 0);
@@ -1497,7 +1507,7 @@ pne_status enumerate_clusters(pne_ctx *ctx, const Geometry &g, int K, int mode, 
     PNE_LAUNCH_CHECK(ctx);
     if (last_bfs >= 1) {
         ProfScope ps__(ctx, s, "enum_emit");
-        launch_expand(kEmit, final_kind == 3, G, s, gv, A, 1, last_bfs, K, mode, out);
+        launch_expand(kEmit, fuse && dfs_level == 0, G, s, gv, A, 1, last_bfs, K, mode, out);
     }
     PNE_LAUNCH_CHECK(ctx);
     if (dfs_level) dfs(A, dfs_level, 1, out);
