@@ -11,14 +11,17 @@ networks.  Metric: PNE terms contracted per second (whole job, all ranks).
                   [--dtype f64|f32|tf32|bf16] [--bp ff|fp64]
                   [--workload random16|ising4|ising3d|batched|serve] [--no-extras]
 
-At one GPU the default run also measures, in the same process and under
-"workloads" of the same JSON line: the step with FP64 BP; the 3D Ising 8x8x8
+At one GPU the default run also measures, in the same process: the step with FP64 BP; the 3D Ising 8x8x8
 networks at orders 8 and 10 in FP64/TF32/BF16 against the closed form; the
 batched form (4096 networks, one fused launch); and the served form against
 the plain FP64 single-request path on the same request trace.
 
 Under torchrun each rank works on its own 32 networks (weak scaling, no
-collective on the data path); rank 0 prints one JSON line.
+collective on the data path).  Rank 0 prints one JSON line with the measurement
+on stdout (short enough to survive whole where only the end of the output is
+kept) and what explains it on stderr, one JSON line per part: host times,
+roofline, variants, peaks and each of the other workloads.  --details FILE writes
+both as one JSON object.
 """
 from __future__ import annotations
 
@@ -274,6 +277,34 @@ class StepBench:
         return total, res, prof
 
 
+# what goes on the one line; of the nested parts only these
+LINE_KEYS = ("impl", "metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step", "higher_is_better", "scaling",
+             "vs_baseline", "dtype", "data", "config", "e2e", "gpu_launches", "clocks", "roofline", "cpu_baseline")
+LINE_PARTS = {"config": ("workload", "networks_per_step_per_gpu", "terms_per_network", "K", "bp_arithmetic", "l2",
+                         "parallelism", "offered_rate_req_s", "trace_s"),
+              "roofline": ("kernel", "bound", "frac"),
+              "cpu_baseline": ("value", "unit", "cores", "kind")}
+
+
+def emit(out, details=""):
+    """The measurement of `out` on one line of stdout, everything else of it on
+    stderr, a line per part; all of it in the file `details` when given."""
+    line = {}
+    for k in LINE_KEYS:
+        if k in out:
+            part = LINE_PARTS.get(k)
+            line[k] = {q: out[k][q] for q in part if q in out[k]} if part else out[k]
+    rest = {k: v for k, v in out.items() if k not in LINE_KEYS or line[k] != v}
+    workloads = rest.pop("workloads", {})
+    for k, v in list(rest.items()) + list(workloads.items()):
+        print(json.dumps({k: v}), file=sys.stderr)
+    sys.stderr.flush()
+    if details:
+        with open(details, "w") as f:
+            json.dump(out, f, indent=1)
+    print(json.dumps(line), flush=True)
+
+
 def main():
     ap = argparse.ArgumentParser()
     ap.add_argument("--gpus", type=int, default=1)
@@ -293,6 +324,7 @@ def main():
                     help="networks per call of the blocked chi = 16 grid contraction workload")
     ap.add_argument("--bp", default="ff", choices=["fp64", "ff"],
                     help="BP sweep arithmetic: FP64, or float-float pairs on the FP32 pipes")
+    ap.add_argument("--details", default="", help="file for the whole record, a JSON object")
     args = ap.parse_args()
     wl = WORKLOADS[args.workload]
 
@@ -305,12 +337,12 @@ def main():
     if wl["kind"] == "batched":
         out = run_batched(args, wl, rank, world, local_rank)
         if rank == 0 and out:
-            print(json.dumps(out))
+            emit(out, args.details)
         return 0
     if wl["kind"] == "serve":
         out = run_serve_workload(args, wl, rank, world, local_rank)
         if rank == 0 and out:
-            print(json.dumps(out))
+            emit(out, args.details)
         return 0 if out else 1
     return run_step_bench(args, wl, rank, world, local_rank)
 
@@ -461,7 +493,7 @@ def run_step_bench(args, wl, rank, world, local_rank):
             extras[name]["bench_seconds"] = round(time.perf_counter() - t0, 1)
         out["workloads"] = extras
     if rank == 0:
-        print(json.dumps(out))
+        emit(out, args.details)
     ctx.close()
     if world > 1:
         dist.destroy_process_group()
