@@ -495,11 +495,10 @@ __global__ void __launch_bounds__(kF64Threads, G > 4 ? 1 : 2) f64_gemm_kernel(F6
 // ---------------------------------------------------------------- grid contraction
 // Site matrices B_v[n = d Nh + h'][k = u Kh + h] = 2^-s_v T_v[l = h, u, r = h', d]
 // per (set, site), rows zero-padded to ldb, in the product's operand type; s_v
-// is the exponent of the tensor's largest |entry|.  A cluster of eight blocks
-// per tensor, each searching an eighth of it and writing an eighth of the rows,
-// a warp per row: at chi = 16 a tensor is 512 KB, and one block each with a
-// division per entry took 0.28 ms for 640 of them, this 0.12.
-constexpr int kSiteBlocks = 8;
+// is the exponent of the tensor's largest |entry|.  gridDim.z blocks per tensor
+// (a cluster when more than one), each searching its part of it and writing its
+// part of the rows, a warp per row; see site_blocks.
+constexpr int kSiteBlocks = 8;                  // most blocks per tensor
 
 template <typename E>
 __device__ __forceinline__ E site_elem(double x);
@@ -511,11 +510,11 @@ template <>
 __device__ __forceinline__ __nv_bfloat16 site_elem<__nv_bfloat16>(double x) { return __float2bfloat16_rn((float)x); }
 
 template <typename E>
-__global__ void __cluster_dims__(1, 1, kSiteBlocks) __launch_bounds__(256)
+__global__ void __launch_bounds__(256)
     grid_sites_kernel(const double *data, int64_t set_stride, const SiteMap *sites, E *Bm, int64_t b_stride,
                       const int64_t *ldb, long long *log2s)
 {
-    const int v = blockIdx.x, set = blockIdx.y, part = blockIdx.z;
+    const int v = blockIdx.x, set = blockIdx.y, part = blockIdx.z, parts = gridDim.z;
     const SiteMap sm = sites[v];
     const double *t = data + set * set_stride + sm.t_off;
     const int Kh = sm.dim[0], Ku = sm.dim[1], Nh = sm.dim[2], Nd = sm.dim[3];
@@ -525,7 +524,7 @@ __global__ void __cluster_dims__(1, 1, kSiteBlocks) __launch_bounds__(256)
     cg::cluster_group cluster = cg::this_cluster();
     // the largest |entry| by its bits (comparing doubles costs FP64 time), a NaN passed over
     unsigned long long mx = 0;
-    for (int64_t i = part * 256 + threadIdx.x; i < n_ent; i += 256 * kSiteBlocks) {
+    for (int64_t i = part * 256 + threadIdx.x; i < n_ent; i += 256 * parts) {
         const unsigned long long bits = (unsigned long long)__double_as_longlong(t[i]) & 0x7fffffffffffffffull;
         if (bits <= 0x7ff0000000000000ull && bits > mx) mx = bits;
     }
@@ -534,23 +533,24 @@ __global__ void __cluster_dims__(1, 1, kSiteBlocks) __launch_bounds__(256)
         if (o > mx) mx = o;
     }
     if ((threadIdx.x & 31) == 0) largest[threadIdx.x >> 5] = mx;
-    cluster.sync();
+    if (parts > 1) cluster.sync();
+    else __syncthreads();
     mx = 0;
-    for (int i = threadIdx.x & 31; i < 8 * kSiteBlocks; i += 32) {
-        const unsigned long long o = cluster.map_shared_rank(largest, i >> 3)[i & 7];
+    for (int i = threadIdx.x & 31; i < 8 * parts; i += 32) {
+        const unsigned long long o = parts > 1 ? cluster.map_shared_rank(largest, i >> 3)[i & 7] : largest[i];
         if (o > mx) mx = o;
     }
     for (int off = 16; off > 0; off >>= 1) {
         const unsigned long long o = __shfl_xor_sync(0xffffffffu, mx, off);
         if (o > mx) mx = o;
     }
-    cluster.sync();                             // no block leaves while its maxima are read
+    if (parts > 1) cluster.sync();              // no block leaves while its maxima are read
     const double top = __longlong_as_double((long long)mx);
     const int e = top > 0.0 ? ilogb(top) : 0;
     const double sc = ldexp(1.0, -e);
     const int ld = (int)ldb[v];
     E *out = Bm + set * b_stride + sm.b_off;
-    for (int n = part * 8 + (threadIdx.x >> 5); n < N; n += 8 * kSiteBlocks) {
+    for (int n = part * 8 + (threadIdx.x >> 5); n < N; n += 8 * parts) {
         const int d = n / Nh, hp = n - d * Nh;
         const double *row = t + (int64_t)hp * sm.stride[2] + (int64_t)d * sm.stride[3];
         for (int k = threadIdx.x & 31; k < ld; k += 32) {
@@ -1211,6 +1211,41 @@ cudaError_t launch_grid_stream(const RingParams<E> &p, int batch, int n_sm, cuda
     return launch_stream<EB, kBoxes>(ma, mb, q, n_sm, s);
 }
 
+// Blocks per tensor of grid_sites_kernel.  One of them works through n entries in
+// about 1.6 ns each, a launch of T tensors takes about 5 ns per block: P blocks a
+// tensor are best near P^2 = n / (3 T).  us of the FP64 launch, 3 x 3 networks, with
+// 1, 2, 4 and 8 blocks: chi 2, 1000 sets 39, 96, 178, 364; chi 7, 1000 sets 74, 142,
+// 240, 445; chi 11, 1 set 32, 33, 22, 16, 300 sets 92, 103, 127, 191; chi 16, 1 set
+// 104, 58, 34, 25, 64 sets 133, 85, 76, 77, 200 sets 292, 157, 150, 190 (one block
+// with a division per entry took 63, 85, 34, 90, 140, 181 and 325).
+int site_blocks(const GridPlan &plan, int nb)
+{
+    int64_t n = 1;
+    for (const GridStep &sd : plan.steps) n = std::max(n, (int64_t)sd.Ku * sd.Kh * sd.Nd * sd.Nh);
+    int P = 1;
+    while (P < kSiteBlocks && n >= 3 * (int64_t)(2 * P) * (2 * P) * plan.n * nb) P *= 2;
+    return P;
+}
+
+template <typename E>
+cudaError_t launch_grid_sites(const GridPlan &plan, int nb, const double *data, int64_t set_stride, const SiteMap *maps,
+                              E *Bm, const int64_t *ldb, long long *lg, cudaStream_t s)
+{
+    const int blocks = site_blocks(plan, nb);
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)plan.n, (unsigned)nb, (unsigned)blocks);
+    cfg.blockDim = dim3(256, 1, 1);
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = 1;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = (unsigned)blocks;
+    cfg.attrs = attr;
+    cfg.numAttrs = blocks > 1 ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, grid_sites_kernel<E>, data, set_stride, maps, Bm, plan.b_total, ldb, lg);
+}
+
 size_t tc_smem_bytes(int BN)
 {
     return (size_t)2 * (kATileBytes + BN * kChunk) + 1024;
@@ -1522,13 +1557,15 @@ pne_status grid_run(pne_ctx *ctx, const GridPlan &plan, const double *data, int6
         auto run_tc = [&](auto tag) -> cudaError_t {
             using E = decltype(tag);
             E *S0 = (E *)dS.ptr, *S1 = (E *)dA.ptr;
+            cudaError_t ee;
             {
                 ProfScope ps(ctx, s, "grid_sites");
                 grid_init_kernel<E><<<ib, 128, 0, s>>>(S0, max_state, mb, lg, nb);
-                grid_sites_kernel<E><<<dim3(n, nb, kSiteBlocks), 256, 0, s>>>(
-                    data, set_stride, (const SiteMap *)dMaps.ptr, (E *)dB.ptr, b_total, (const int64_t *)dLdb.ptr, lg);
+                ee = cudaGetLastError();
+                if (ee == cudaSuccess)
+                    ee = launch_grid_sites<E>(plan, nb, data, set_stride, (const SiteMap *)dMaps.ptr, (E *)dB.ptr,
+                                              (const int64_t *)dLdb.ptr, lg, s);
             }
-            cudaError_t ee = cudaGetLastError();
             if (ee != cudaSuccess) return ee;
             for (int v = 0; v < n; ++v) {
                 const GridStep &sd = plan.steps[(size_t)v];
@@ -1566,10 +1603,12 @@ pne_status grid_run(pne_ctx *ctx, const GridPlan &plan, const double *data, int6
         {
             ProfScope ps(ctx, s, "grid_sites");
             grid_init_kernel<double><<<ib, 128, 0, s>>>(S0, max_state, mb, lg, nb);
-            grid_sites_kernel<double><<<dim3(n, nb, kSiteBlocks), 256, 0, s>>>(
-                data, set_stride, (const SiteMap *)dMaps.ptr, (double *)dB.ptr, b_total, (const int64_t *)dLdb.ptr, lg);
+            e = cudaGetLastError();
+            if (e == cudaSuccess)
+                e = launch_grid_sites<double>(plan, nb, data, set_stride, (const SiteMap *)dMaps.ptr, (double *)dB.ptr,
+                                              (const int64_t *)dLdb.ptr, lg, s);
         }
-        if ((e = cudaGetLastError()) != cudaSuccess) return fail(e, "grid site matrices");
+        if (e != cudaSuccess) return fail(e, "grid site matrices");
         for (int v = 0; v < n; ++v) {
             const GridStep &sd = plan.steps[(size_t)v];
             F64Params p{};
