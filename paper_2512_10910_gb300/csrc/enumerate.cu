@@ -346,7 +346,7 @@ __global__ void widen_counts_kernel(const int32_t *row0, const int64_t *lv, int 
 // whose children would not fit stops the search (ctl->stop = d, ctl->need =
 // the size it asked for) and every deeper level is left empty.  Count and
 // slot tables are [K+1][cap], indexed by arena position; with the closing
-// step (LOOP mode, K >= 4) a node of level t emits size t + 1 only, except
+// step (LOOP mode, K >= 3) a node of level t emits size t + 1 only, except
 // the last level's, which emit sizes K - 2, K - 1 and K, so three rows hold
 // the counts in output order: row 0 every level's own size (levels ascend
 // with the arena position), rows 1 and 2 the last level's K - 1 and K.  On
@@ -588,7 +588,7 @@ __device__ __forceinline__ void sort_regs(int32_t (&x)[N])
         }
 }
 
-// Writes the cluster S + e0 (+ e1, e2 when >= 0) of a node: bonds and vertices
+// Writes the cluster S + e1 (+ e0, e2 when >= 0) of a node: bonds and vertices
 // (the node's list plus b0, b1 when >= 0) sorted ascending, rows padded with -1.
 __device__ void write_child_cluster(const Emit &o, int64_t slot, const Node &nd, int e0, int e1, int e2, int b0, int b1)
 {
@@ -597,8 +597,8 @@ __device__ void write_child_cluster(const Emit &o, int64_t slot, const Node &nd,
     int32_t sv[NS], vv[NVx];
 #pragma unroll
     for (int q = 0; q < kPrefixMax; ++q) sv[q] = q < t ? nd.S[q] : INT_MAX;
-    sv[kPrefixMax] = e0;
-    sv[kPrefixMax + 1] = e1 >= 0 ? e1 : INT_MAX;
+    sv[kPrefixMax] = e0 >= 0 ? e0 : INT_MAX;
+    sv[kPrefixMax + 1] = e1;
     sv[kPrefixMax + 2] = e2 >= 0 ? e2 : INT_MAX;
 #pragma unroll
     for (int q = 0; q < kNodeV; ++q) vv[q] = q < vn ? nd.vv[q] : INT_MAX;
@@ -606,7 +606,7 @@ __device__ void write_child_cluster(const Emit &o, int64_t slot, const Node &nd,
     vv[kNodeV + 1] = b1 >= 0 ? b1 : INT_MAX;
     sort_regs(sv);
     sort_regs(vv);
-    const int s = t + 1 + (e1 >= 0 ? 1 : 0) + (e2 >= 0 ? 1 : 0), n = vn + (b0 >= 0 ? 1 : 0) + (b1 >= 0 ? 1 : 0);
+    const int s = t + 1 + (e0 >= 0 ? 1 : 0) + (e2 >= 0 ? 1 : 0), n = vn + (b0 >= 0 ? 1 : 0) + (b1 >= 0 ? 1 : 0);
     int32_t *er = o.edges + slot * o.width;
 #pragma unroll
     for (int q = 0; q < NS; ++q)
@@ -716,7 +716,7 @@ __device__ void close_child(const GeomView &g, const Node &nd, const NodeTabs &T
                 const int z = __shfl_up_sync(0xffffffffu, incl, off);
                 if (lane >= off) incl += z;
             }
-            const int ec = nd.U[io];
+            const int ec = io >= 0 ? nd.U[io] : -1;
             if (emit) write_child_cluster(out, slotA + nA + __popc(em & lt), nd, ec, C.e[i], -1, cb, b2);
             int64_t slot = slotB + nB + (incl - np);
             for (uint64_t m = close; m; m &= m - 1)
@@ -733,8 +733,9 @@ __device__ void close_child(const GeomView &g, const Node &nd, const NodeTabs &T
 // The block's chunk of the node range [r0, r1).  kChildren writes the
 // children from arena slot next + cbase_chunk on (cbase_chunk: the children of
 // the chunks before this one).
-// With FUSE (LOOP mode, K >= 4) the tables have the three rows of the closing
-// step, and nodes of size K - 3 close their children themselves.
+// With FUSE (LOOP mode, K >= 3) the tables have the three rows of the closing
+// step, and nodes of size K - 3 close their children themselves; at K = 3 a node of
+// size 1 closes itself (16 x 16, K = 3: 86 us a search, 107 through a second level).
 // One instance per pass keeps each kernel's code small enough for the
 // instruction cache.
 template <int PASS, bool FUSE>
@@ -743,13 +744,14 @@ __device__ void expand_chunk(const GeomView &g, const Arena &A, int64_t r0, int6
 {
     constexpr int pass = PASS;
     constexpr bool fuse = FUSE;
+    constexpr bool closes_self = pass == kClose || (pass == kEmit && fuse);
     __shared__ Node sh_node[kExpandWarps];
     __shared__ int32_t sh_a[kExpandWarps][kNodeU], sh_b[kExpandWarps][kNodeU];
     __shared__ int32_t sh_ia[kExpandWarps][kNodeU], sh_ib[kExpandWarps][kNodeU];
     __shared__ uint64_t sh_tmask[kExpandWarps][kNodeV];
     __shared__ int32_t sh_tw[kExpandWarps][kNodeU];
     __shared__ int32_t sh_stage[kExpandWarps][32 * kStageWords];
-    __shared__ int32_t sh_close[kExpandWarps][(pass == kClose || (pass == kEmit && fuse)) ? 4 * kNodeU + kMaxNew : 1];
+    __shared__ int32_t sh_close[kExpandWarps][closes_self ? 4 * kNodeU + kMaxNew : 1];
     __shared__ int64_t wsum[kExpandWarps];
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const unsigned lt = (1u << lane) - 1u;
@@ -773,7 +775,7 @@ __device__ void expand_chunk(const GeomView &g, const Arena &A, int64_t r0, int6
         if (pass == kChildren) want = __ldcg(reinterpret_cast<const unsigned long long *>(A.gmask + u));
         else if (pass == kEmit) want = __ldcg(reinterpret_cast<const unsigned long long *>(A.emask + u));
         uint64_t closes = 0;                             // children with a cluster of size K - 1 or K below them
-        if (pass == kEmit && fuse && __ldcg(&A.nodes[u].t) == K - 3)
+        if (pass == kEmit && fuse && __ldcg(&A.nodes[u].t) == max(K - 3, 1))
             closes = __ldcg(reinterpret_cast<const unsigned long long *>(A.gmask + u));
         if ((want | closes) == 0) continue;
         // L2 loads: these nodes were written by other blocks
@@ -794,7 +796,8 @@ __device__ void expand_chunk(const GeomView &g, const Arena &A, int64_t r0, int6
         const uint32_t dmask = __ballot_sync(0xffffffffu, lane < vn && nd.vd[lane] == 1);
         __syncwarp();
         constexpr bool closing_children = pass == kClose;
-        if (pass == kCount || pass == kClose) {
+        const bool self = closes_self && K == 3;         // the node is itself the set of size K - 2
+        if ((pass == kCount || pass == kClose) && !self) {
             // the candidates at each vertex of the node
             for (int k = 0; k < vn; ++k) {
                 const unsigned m0 = __ballot_sync(0xffffffffu, lane < nU && (T.ia[lane] == k || T.ib[lane] == k));
@@ -837,7 +840,8 @@ __device__ void expand_chunk(const GeomView &g, const Arena &A, int64_t r0, int6
             int32_t NU[kMaxNew], NB[kMaxNew];
             int nn = 0;
             Child c{-1, -1, -1, 0u, 0};
-            const bool mine = i < nU && (((want | closes) >> i) & 1);
+            const bool mine = i < nU && !self && (((want | closes) >> i) & 1);
+            if (self) grow = i == 0;
             if (mine) {
                 c = make_child(T, i, dmask);
                 const int e = nd.U[i];
@@ -913,15 +917,15 @@ __device__ void expand_chunk(const GeomView &g, const Arena &A, int64_t r0, int6
                 __syncwarp();
             }
             if (pass == kEmit && emit)
-                write_child_cluster(out, ebase + n_emit + __popc(em & lt), nd, nd.U[i], -1, -1, c.b, -1);
-            if constexpr (pass == kClose || (pass == kEmit && fuse)) {
+                write_child_cluster(out, ebase + n_emit + __popc(em & lt), nd, -1, nd.U[i], -1, c.b, -1);
+            if constexpr (closes_self) {
                 // the children that may still close, one after another
-                const uint32_t cdm = c.dmask | (c.b >= 0 ? 1u << vn : 0u);
+                const uint32_t cdm = self ? dmask : c.dmask | (c.b >= 0 ? 1u << vn : 0u);
                 unsigned done = 0;
                 for (unsigned rem = closer ? gm : 0u; rem; rem &= rem - 1) {
                     const int o = __ffs(rem) - 1;
                     int nno = __shfl_sync(0xffffffffu, nn, o);
-                    const int io = i0 + o;
+                    const int io = self ? -1 : i0 + o;
                     if (lane == o)
                         for (int q = 0; q < nn; ++q) C.nu[q] = NU[q];
                     __syncwarp();
@@ -1352,10 +1356,10 @@ pne_status enumerate_clusters(pne_ctx *ctx, const Geometry &g, int K, int mode, 
     if ((kPrefixMax + 1) * (maxdeg - 1) > kNodeU) { set_error(ctx, PNE_EINVAL, "site degree too large"); return PNE_EINVAL; }
     GeomView gv{g.d_bond_site, g.d_site_ptr, g.d_site_bonds, g.d_site_nbr};
     // prefix levels 1..D are expanded breadth-first; the last one closes the
-    // three remaining sizes (LOOP mode, D == K - 3), only emits (D == K - 1) or
+    // three remaining sizes (LOOP mode, D == K - 3, or the two above 1 at K == 3), only emits (D == K - 1) or
     // is searched depth-first (K - 1 > kPrefixMax)
-    const bool fuse = mode == PNE_MODE_LOOP && K >= 4 && K - 3 <= kPrefixMax;
-    const int D = fuse ? K - 3 : ((K <= 1) ? 1 : std::min(kPrefixMax, K - 1));
+    const bool fuse = mode == PNE_MODE_LOOP && K >= 3 && K - 3 <= kPrefixMax;
+    const int D = fuse ? std::max(K - 3, 1) : ((K <= 1) ? 1 : std::min(kPrefixMax, K - 1));
     const int final_kind = fuse ? 3 : ((K <= 1) ? 0 : (D == K - 1 ? 1 : 2));
     const bool small = (K <= 12 && umax_need <= 64);
     // chunks of the blocked passes: one wave of resident blocks (the occupancy
