@@ -178,13 +178,12 @@ __device__ __forceinline__ uint32_t to_tf32(float x)
 
 // ---------------------------------------------------------------- the GEMMs
 // C[b][m][n] = sum_k A[b][m][k] B[b][n][k]  (A and B K-major, C row-major)
-template <typename T>
 struct GemmParams {
-    const T *A;
+    const float *A;
     int64_t lda, strideA;
-    const T *B;
+    const float *B;
     int64_t ldb, strideB;
-    T *C;
+    float *C;
     int64_t ldc, strideC;
     int M, N, K;
     int *err;   // set to 1 when a bounded wait gave up
@@ -223,7 +222,7 @@ __device__ __forceinline__ uint32_t tile_off(int r, int c)
 }
 
 template <int EB>
-__global__ void __launch_bounds__(kTcThreads, 1) tc_gemm_kernel(GemmParams<float> p, int BN)
+__global__ void __launch_bounds__(kTcThreads, 1) tc_gemm_kernel(GemmParams p, int BN)
 {
     extern __shared__ uint8_t smem_raw[];
     __shared__ __align__(8) uint64_t mbar[2];
@@ -1254,7 +1253,7 @@ size_t tc_smem_bytes(int BN)
 // pne_dense_gemm on the persistent kernel, B rounded into `W` first; used =
 // false when A cannot be described to the copy engine
 template <int EB>
-cudaError_t launch_dense_stream(const GemmParams<float> &p, int batch, int n_sm, void *W, int64_t ldw, cudaStream_t s,
+cudaError_t launch_dense_stream(const GemmParams &p, int batch, int n_sm, void *W, int64_t ldw, cudaStream_t s,
                                 bool &used)
 {
     used = false;
@@ -1303,7 +1302,7 @@ __global__ void pad_rows_kernel(const float *A, int64_t lda, int64_t strideA, in
 constexpr int64_t kPadBytes = (int64_t)96 << 20;
 
 template <int EB>
-cudaError_t launch_padded_stream(const GemmParams<float> &p, int batch, int n_sm, float *P, int64_t ldp, void *W,
+cudaError_t launch_padded_stream(const GemmParams &p, int batch, int n_sm, float *P, int64_t ldp, void *W,
                                  int64_t ldw, cudaStream_t s, bool &used)
 {
     const int64_t most = std::max<int64_t>(kPadBytes / (ldp * 4) / kTcBM * kTcBM, kTcBM);
@@ -1312,7 +1311,7 @@ cudaError_t launch_padded_stream(const GemmParams<float> &p, int batch, int n_sm
     for (int b = 0; b < batch; b += sets)
         for (int64_t m = 0; m < p.M; m += rows) {
             const int nb = std::min(sets, batch - b);
-            GemmParams<float> q = p;
+            GemmParams q = p;
             q.M = (int)std::min<int64_t>(rows, p.M - m);
             q.A = P;
             q.lda = ldp;
@@ -1330,7 +1329,7 @@ cudaError_t launch_padded_stream(const GemmParams<float> &p, int batch, int n_sm
 }
 
 template <int EB>
-cudaError_t launch_tc(pne_ctx *ctx, const GemmParams<float> &p, int batch, cudaStream_t s)
+cudaError_t launch_tc(pne_ctx *ctx, const GemmParams &p, int batch, cudaStream_t s)
 {
     const bool aligned = (reinterpret_cast<uintptr_t>(p.A) & 15) == 0 && p.lda % 4 == 0 &&
                          (batch == 1 || (p.strideA % 4 == 0 && p.strideA > 0));
@@ -1708,7 +1707,7 @@ pne_status pne_dense_gemm(pne_ctx *ctx, pne_dtype dtype, int32_t batch, int32_t 
             p.K = K;
             e = launch_f64<false>(p, batch, ctx->n_sm, s);
         } else {
-            GemmParams<float> p{(const float *)A, lda, strideA, (const float *)B, ldb, strideB, (float *)C, ldc,
+            GemmParams p{(const float *)A, lda, strideA, (const float *)B, ldb, strideB, (float *)C, ldc,
                                 strideC, M, N, K, flag ? flag : (int *)err.ptr};
             e = dtype == PNE_TF32 ? launch_tc<4>(ctx, p, batch, s) : launch_tc<2>(ctx, p, batch, s);
         }
