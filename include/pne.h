@@ -455,7 +455,7 @@ void pne_weights_destroy(pne_weights *w);
  * exp(-log_scale) (k = |x| for form 1, k = position in Eq. A4 for form 0),
  * n_terms.  Partition bonds as in pne_enumerate_combinatorial.  Limits: M <=
  * 20, 1 <= rank < every partitioned bond's dimension, an intermediate tensor
- * of at most 2^20 entries (PNE_EINVAL otherwise).  Synchronises `stream`. */
+ * of at most 2^18 entries (PNE_EINVAL otherwise).  Synchronises `stream`. */
 pne_status pne_rank_r_expand(pne_ctx *ctx, const pne_weights *w, int32_t rank, int32_t form, int32_t n_partitions,
                              const int32_t *partition_ptr, const int32_t *partition_bonds, void *stream,
                              pne_result *out);

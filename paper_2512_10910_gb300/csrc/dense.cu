@@ -17,8 +17,10 @@
 // The large products run on one persistent kernel (tc_stream_kernel: operand
 // stages filled by the Tensor Memory Accelerator, tcgen05.mma with M = 128,
 // N <= 256 and FP32 accumulation in tensor memory, a finished tile stored while
-// the next accumulates).  Small products of pne_dense_gemm, and those whose A
-// is not on 16-byte boundaries, take tc_gemm_kernel: one CTA per tile, K staged
+// the next accumulates); products whose A is not on 16-byte boundaries get there
+// behind a padded copy of A where many columns repay it (launch_padded_stream).
+// Small products of pne_dense_gemm, and the unaligned ones that are shallow or
+// narrow (launch_tc has the rule), take tc_gemm_kernel: one CTA per tile, K staged
 // 128 bytes per row at a time in two shared-memory stages written by all
 // threads in the canonical no-swizzle K-major layout (8-row x 16-byte core
 // matrices, the two core matrices of one MMA K step 128 bytes apart, 8-row
@@ -624,9 +626,10 @@ struct RingParams {
 // byte of A and C against 140 at the TF32 and 290 at the BF16 tensor rate), so
 // the split is chosen to keep loads in flight: one block per SM walks the
 // tiles; one thread issues the loads (64 KB of A in flight per SM), one the
-// MMAs, four warps store a finished tile from tensor memory while the next one
-// accumulates in its other half; the stages fill the shared memory, up to 12
-// (with four, the N = 16 steps of the last column read 4.1 TB/s).  An operand row of a stage is 128 bytes, copied
+// MMAs, eight warps (four where A is rounded, see store_warps) store a finished
+// tile from tensor memory while the next one accumulates in its other half; the
+// stages fill the shared memory, up to 12 (with four, the N = 16 steps of the last
+// column read 4.1 TB/s).  An operand row of a stage is 128 bytes, copied
 // in boxes of the widest swizzle whose bytes are contiguous in A (128, 64 or
 // 32; 16 without one): boxes of 16 bytes, which every stage used before, cost
 // the copy engine one request per 16 bytes and bound the kernel.

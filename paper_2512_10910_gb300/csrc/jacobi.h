@@ -36,8 +36,10 @@ __device__ __forceinline__ double widen(float x)        // normal x
 // the error left is t^2 / (1 + t^2) times its square each time, 2^-45 and below
 // FP64's rounding.  The second step matters although the first leaves columns
 // that the next sweep would still rotate: an inner product just above the bound
-// is rotated once and never again, and a small entry of V is a few such t (2.1e-14
-// of its own size with one step, 4.1e-16 with two, as with division and root).
+// is rotated once and never again, and a small entry of V is a few such t (a sine is
+// off by up to 1.5e-14 of its own size with one step, 3.9e-16 with two, 4.3e-16 with
+// division and root).  Weight passing of eight 3 x 3 networks of chi = 16 takes 99 ms
+// with two steps, 95 with one.
 __device__ __forceinline__ void jacobi_rotation(double a, double b, double g, double &cs, double &sn)
 {
     const double h = b - a;

@@ -279,9 +279,9 @@ __device__ __forceinline__ int wp_parts(int rest) { return min(kWpParts, (rest +
 // its rows.  FP64 multiply-adds bound the large tensors (two per clock and
 // SM: 2 x 1.05 M for a 16^4 tensor, so the split over SMs is what pays), the
 // chain of column steps and Jacobi rounds the small ones.
-// Measured, blocked Ising 3 x 3, 8 sets, 0.65 to 0.8 T_c: chi = 16 860 -> 93 ms
+// Measured, blocked Ising 3 x 3, 8 sets, 0.65 to 0.8 T_c: chi = 16 933 -> 99 ms
 // (one block of 256 threads per set walked each matrix column by column in L2
-// and rotated one pair of columns at a time), chi = 8 246 -> 46, chi = 4 89 -> 30.
+// and rotated one pair of columns at a time), chi = 8 264 -> 52, chi = 4 97 -> 31.
 template <int DM>
 __global__ void __launch_bounds__(kWpThreads) weight_passing_kernel(WPParams p, int blocks)
 {
@@ -915,8 +915,8 @@ pne_status pne_weight_passing(pne_ctx *ctx, const pne_network *net, double alpha
     for (int b = 0; b < g.n_bonds; ++b) dmax = std::max(dmax, (int)g.bond_dim[b]);
     // Blocks per set: two take the two sides of a bond, more share the rows of
     // tensors above one panel, while every set's cluster fits the GPU at once.
-    // 3 x 3, chi = 16, 8 sets: 189, 124, 104 and 93 ms with 1, 2, 4 and 8 blocks;
-    // chi = 8 (512 rows): 64, 46.3, 45.7, 45.7.
+    // 3 x 3, chi = 16, 8 sets: 212, 132, 110 and 99 ms with 1, 2, 4 and 8 blocks;
+    // chi = 8 (512 rows, one panel): 73 and 52 with 1 and 2.
     int blocks = 1;
     const int most = tmax / dmax > kWpPanel ? kWpCluster : 2;
     while (2 * blocks <= most && 2 * blocks * B <= ctx->n_sm) blocks *= 2;
