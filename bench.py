@@ -569,10 +569,10 @@ def step_roofline(args, pne, ctx, ctypes_stream, g, sb, res, prof, prof_steps, B
                          f"({launches // prof_steps} launches of {fam} per search)")
         if args.workload == "random16":
             # what bounds it: issue slots and the integer pipe, per launch (ncu)
-            roof.update(issue={"expand_kernel": {"issue_active_pct": 23.4, "alu_pipe_pct": 20.9,
-                                                 "dram_bytes_per_launch": 0.77e6},
-                               "expand_children_kernel": {"issue_active_pct": 12.9, "alu_pipe_pct": 8.7,
-                                                          "dram_bytes_per_launch": 0.49e6},
+            roof.update(issue={"expand_kernel": {"issue_active_pct": 20.4, "alu_pipe_pct": 19.0,
+                                                 "dram_bytes_per_launch": 0.26e6},
+                               "expand_children_kernel": {"issue_active_pct": 11.7, "alu_pipe_pct": 7.8,
+                                                          "dram_bytes_per_launch": 0.31e6},
                                "source": "ncu smsp__issue_active, sm__pipe_alu_cycles_active, dram__bytes_*, "
                                          "averages over the launches of one step, this workload"})
     if roof["achieved"] is not None and roof["peak"]:
