@@ -20,7 +20,7 @@
 // strip (chi -> chi) as its other shapes.  One thread per (p, s) keeps the
 // chi^2 inputs of its fibre in registers and the matrix in shared memory (a
 // broadcast read); consecutive threads take consecutive s, so the fibre's
-// loads coalesce whenever S >= 32.  Every multiply-add is FP64.
+// loads coalesce whenever S >= 32.  Multiply-adds are FP64 or float-float (ff_dot).
 //
 // The power iteration keeps the vector unnormalised with a per-tensor scale;
 // the reduction of each iteration forms |w|^2, <v, w> (the Rayleigh quotient
